@@ -373,7 +373,7 @@ int irls_best_shift_error(irls_plan plan, const float* d_U, const float* d_Xu, f
  * cudaMalloc's implicit device synchronisation or an out-of-memory failure after start-up.
  * It computes what irls_precond_laplacian computes with IRLS_PREC_FP32, d_Z = L^+ (tau d_R), but
  * needs no plan and allocates nothing: the DCT bases and intermediates live in one fixed
- * 1.84 MB buffer compiled into the library (every GPU that loads the library holds it until the
+ * 1.05 MB buffer compiled into the library (every GPU that loads the library holds it until the
  * process exits), sized for H, W <= IRLS_NOALLOC_MAX_SIDE.
  *   d_R, d_Z  H x W float32 device arrays, row-major and contiguous, owned by the caller;
  *   tau       > 0 (the penalty of the plan-based form);

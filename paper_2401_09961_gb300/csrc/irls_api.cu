@@ -1318,6 +1318,11 @@ int irls_precond_laplacian(irls_plan p, const float* R, float* Z, void* stream) 
     try {
         DeviceGuard g(p->dev);
         StencilArgs a = make_args(p);
+        // the float32 dense products read and write rows of any pitch
+        if (p->opts.precision == IRLS_PREC_FP32 && !p->dct.fft) {
+            ck(dct_apply(p->dct, R, Z, p->W, p->st, 0, a, p->partials, 0, s));
+            return IRLS_OK;
+        }
         ck(cudaMemsetAsync(p->P.rU, 0, p->L.plane_bytes, s));
         ck(launch_copy_in(R, p->H, p->W, p->P.rU, p->ld, s));
         if (a.r16) ck(launch_emit16(p->P.rU, p->H, p->W, p->ld, a.r16, a.r16lo, a.ld16, s));

@@ -129,10 +129,10 @@ struct DctPlan {
     int H, W, Hp, Wp;
     int prec;
     float tau;
-    // fp32 bases: P_N (Hp x Hp) with P_N[i][k], its transpose, and the same for M (may alias N)
-    float *PN, *PNT, *PM, *PMT;
+    // fp32 basis halves of the two sides (dct.cu; may alias when H = W)
+    float *halvesN, *halvesM;
     float *lamN, *lamM;     // eigenvalues, padded with zeros
-    float *T1, *T2;         // fp32 intermediates (Wp x Hp each, reused)
+    float *T1, *T2;         // fp32 intermediates (Wp x Hp each)
     // bfloat16 copies for the tensor-core path (the *lo parts only in split precision)
     void *PN16, *PNT16, *PM16, *PMT16;
     void *PN16lo, *PNT16lo, *PM16lo, *PMT16lo;

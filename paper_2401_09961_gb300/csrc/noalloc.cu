@@ -20,9 +20,9 @@ void set_last_cuda_error(int code);
 namespace {
 
 constexpr int kMaxSide = IRLS_NOALLOC_MAX_SIDE;
-// bases P_N, P_N^T, P_M, P_M^T, two intermediates and the pitched input: seven planes of
-// kMaxSide^2 floats, plus two eigenvalue vectors (1.84 MB for kMaxSide = 256)
-constexpr size_t kScratchFloats = 7u * kMaxSide * kMaxSide + 2u * kMaxSide;
+// the basis halves of two sides and two intermediates: four planes of kMaxSide^2 floats, plus two
+// eigenvalue vectors (1.05 MB for kMaxSide = 256)
+constexpr size_t kScratchFloats = 4u * kMaxSide * kMaxSide + 2u * kMaxSide;
 
 // The scratch itself.  Every device that loads the library holds it until the process exits.
 // In host code this name is only a host-side stand-in: kernels get its device address, looked
