@@ -173,8 +173,8 @@ int irls_plan_dct_form(irls_plan plan);
 
 /* Tile shapes of the CG direction and update kernels (Alg. 2's two stencil passes per
  * iteration, both bound by HBM bandwidth): image rows per thread block, 8 to 64 for a plan
- * (defaults 24 and 32; batches: one of 8, 16, 24, 32, see irls_batch_set_tiles).  They change
- * the block decomposition, so results change within rounding (the reductions' summation order
+ * (defaults 24 and 32; batches: one of 8, 16, 24, 32, see irls_batch_set_tiles), or fewer where
+ * a small image's launch would otherwise leave SMs idle.  They change the block decomposition, so results change within rounding (the reductions' summation order
  * follows the blocks), never the method.  irls_plan_set_tiles sets them (0 keeps a value;
  * anything outside 8..64 is IRLS_ERR_ARG); irls_plan_get_tiles reads the values in use.
  * irls_plan_autotune times, for each kernel, 8, 16, 24 and 32 rows and the row counts that make

@@ -179,7 +179,8 @@ struct irls_plan_s {
     int schedule_stop = 0;
     int dir_rows = 0, upd_rows = 0;   // stencil tile shapes (0: the defaults)
     int rw_rows = 0, fin_rows = 0;    // reweighting and finalize rows (aux_rows of H, W)
-    int sdir_rows = 0, supd_rows = 0; // U-only direction and update rows (whole waves, or 0)
+    int sdir_rows = 0, supd_rows = 0; // U-only direction and update rows (whole waves)
+    int dir_wave = 0, upd_wave = 0;   // one-wave rows of the direction and update kernels
     cudaEvent_t ev[2] = {nullptr, nullptr};
     Profiler prof;
 };
@@ -230,6 +231,8 @@ StencilArgs make_args(const irls_plan_s* p) {
     a.fin_rows = p->fin_rows;
     a.sdir_rows = p->sdir_rows;
     a.supd_rows = p->supd_rows;
+    a.dir_wave = p->dir_wave;
+    a.upd_wave = p->upd_wave;
     return a;
 }
 
@@ -507,7 +510,14 @@ void layout_vec_blocks(irls_batch_s* b) {
     int vblk = 0, ublk = 0, rblk = 0, fblk = 0;
     for (int t = 0; t < b->T; ++t) {
         TileRec& r = b->recs[t];
-        vec_dims(b->H[t], b->W[t], b->dir_rows, b->upd_rows, r.vgx, r.vgy, r.ugy);
+        StencilArgs& a = r.a;
+        a.dir_unit = unit_rows(b->dir_rows, a.dir_wave);
+        a.upd_unit = unit_rows(b->upd_rows, a.upd_wave);
+        a.dir_rows = batch_rows(b->dir_rows, a.dir_wave);
+        a.upd_rows = batch_rows(b->upd_rows, a.upd_wave);
+        r.vgx = vec_blocks_x(b->W[t]);
+        r.vgy = (b->H[t] + a.dir_rows - 1) / a.dir_rows;
+        r.ugy = (b->H[t] + a.upd_rows - 1) / a.upd_rows;
         r.vblk0 = vblk;
         r.ublk0 = ublk;
         r.rblk0 = rblk;
@@ -538,8 +548,8 @@ void drop_graphs(irls_batch_s* b) {
 // one chunk of n batched CG iterations followed by the count of images still iterating
 void issue_chunk(irls_batch_s* b, int n, int slot, cudaStream_t s) {
     for (int c = 0; c < n; ++c) {
-        ck(launch_direction_batched(b->d_recs, b->T, b->total_vec, b->dir_rows, s));
-        ck(launch_update_batched(b->d_recs, b->T, b->total_upd, b->upd_rows, s));
+        ck(launch_direction_batched(b->d_recs, b->T, b->total_vec, s));
+        ck(launch_update_batched(b->d_recs, b->T, b->total_upd, s));
         ck(batch_dct_apply(b->dct, s));
     }
     ck(launch_count_active(b->states, b->T, b->d_count + slot, s));
@@ -712,8 +722,10 @@ int irls_plan_create(int H, int W, const irls_opts* opts, irls_plan* out) {
         p->H = H; p->W = W; p->ld = row_pitch(W);
         p->rw_rows = aux_rows(2, H, W);
         p->fin_rows = aux_rows(3, H, W);
-        p->sdir_rows = wave_rows(4, H, W, kMaxTileRows);
-        p->supd_rows = wave_rows(5, H, W, kMaxTileRows);
+        p->dir_wave = one_wave_rows(0, H, W);
+        p->upd_wave = one_wave_rows(1, H, W);
+        p->sdir_rows = aux_rows(4, H, W);
+        p->supd_rows = aux_rows(5, H, W);
         p->opts = o;
         p->prec_alloc = o.precision;
         p->L = layout(H, W, o.precision);
@@ -1150,6 +1162,8 @@ int irls_batch_create(int ntiles, const int* H, const int* W, const irls_opts* o
             a.prec = o.precision;
             a.rw_rows = aux_rows(2, H[t], W[t]);
             a.fin_rows = aux_rows(3, H[t], W[t]);
+            a.dir_wave = one_wave_rows(0, H[t], W[t]);
+            a.upd_wave = one_wave_rows(1, H[t], W[t]);
             // the direct form reads the update kernel's bf16 copy of r_U; the folded form folds
             // r_U itself
             if (!fold) {
@@ -1242,9 +1256,9 @@ int irls_batch_autotune(irls_batch b, float* h_ms, void* stream) {
                     ck(cudaMemsetAsync(b->states, 0, (size_t)b->T * sizeof(DevState), s));
                     ck(cudaEventRecord(e0, s));
                     if (k == 0)
-                        ck(launch_direction_batched(b->d_recs, b->T, b->total_vec, b->dir_rows, s));
+                        ck(launch_direction_batched(b->d_recs, b->T, b->total_vec, s));
                     else
-                        ck(launch_update_batched(b->d_recs, b->T, b->total_upd, b->upd_rows, s));
+                        ck(launch_update_batched(b->d_recs, b->T, b->total_upd, s));
                     ck(cudaEventRecord(e1, s));
                     ck(cudaEventSynchronize(e1));
                     float t = 0.f;

@@ -114,7 +114,26 @@ struct StencilArgs {
     int dir_rows, upd_rows;
     int rw_rows, fin_rows;
     int sdir_rows, supd_rows;   // U-only system's direction and update kernels (0: 24)
+    // rows that make the direction and update launches of this image one wave (0: unknown): a
+    // launch sums its inner products in units of min(dir_rows, dir_wave) rows, and a single
+    // image's blocks hold one unit (see unit_rows)
+    int dir_wave, upd_wave;
+    int dir_unit, upd_unit;     // batches: rows of a summation unit (dir_rows, upd_rows: of a block)
 };
+
+// Rows of a summation unit for a tile of `rows` rows and a one-wave count of `wave` rows, and the
+// whole units a batch's block holds.  Small images leave most SMs idle at the tile's rows, and a
+// block's rows are a serial chain of about a microsecond each: blocks of the fewest rows that
+// still run at once are as fast as the chip allows.  In a batch the other images fill the chip,
+// and blocks of several units save the halo rows and the block ends.  Measured (us of one launch,
+// direction / update): 1024^2 at 12 rows 30 / 28, at 8 24 / 24, at the one-wave 3 / 4 rows 18 / 22,
+// at 1 28 / 42; 256^2 at 8 rows 22 / 18, at 1 (one wave) 10 / 14; 2048^2 at 24 / 32 rows 53 / 68, at
+// the one-wave 11 / 14 49 / 59.
+inline int unit_rows(int rows, int wave) { return wave > 0 && wave < rows ? wave : rows; }
+inline int batch_rows(int rows, int wave) {
+    const int u = unit_rows(rows, wave);
+    return rows / u * u;
+}
 
 // Image rows per block the CG direction and update kernels are built for, and the defaults
 // (measured fastest at 4096 x 4096).
@@ -223,6 +242,10 @@ int stencil_grid_blocks(int H, int W);
 // 2 reweighting, 3 finalize, 4 and 5 the U-only system's direction and update) on an H x W image a whole number of waves on the current device,
 // between kMinTileRows and `max_rows` (0 when no count in that range does)
 int wave_rows(int kernel, int H, int W, int max_rows);
+// the fewest rows per block (1 or more) with which that launch is a single wave (0: unknown)
+int one_wave_rows(int kernel, int H, int W);
+// blocks of the widest launch whose rows one_wave_rows chose (128-thread blocks, at most 16 an SM)
+constexpr int kMaxWaveBlocks = 16 * 160;
 // rows per block of the reweighting (kernel 2) or finalize (kernel 3) launch for an H x W image:
 // the count of the fewest whole waves up to kMaxTileRows rows, else kDefaultUpdRows.  A single-image plan and a batch
 // both take it, so that they sum in the same order.
@@ -249,14 +272,12 @@ cudaError_t launch_adj_final(const Planes& P, const StencilArgs& a, const float*
 // batched launches over a device array of TileRec (one launch for all images; images whose CG
 // run has stopped return at once)
 void strip_dims(int H, int W, int& gx, int& gy);
-void vec_dims(int H, int W, int dir_rows, int upd_rows, int& gx, int& gy_dir, int& gy_upd);
+int vec_blocks_x(int W);
 cudaError_t launch_init_batched(const TileRec* recs, int T, int total_strip, cudaStream_t s);
 cudaError_t launch_bnorm_batched(const TileRec* recs, int T, int total_strip, cudaStream_t s);
 cudaError_t launch_reweight_batched(const TileRec* recs, int T, int total_rw, cudaStream_t s);
-cudaError_t launch_direction_batched(const TileRec* recs, int T, int total_vec, int rows,
-                                     cudaStream_t s);
-cudaError_t launch_update_batched(const TileRec* recs, int T, int total_upd, int rows,
-                                  cudaStream_t s);
+cudaError_t launch_direction_batched(const TileRec* recs, int T, int total_vec, cudaStream_t s);
+cudaError_t launch_update_batched(const TileRec* recs, int T, int total_upd, cudaStream_t s);
 cudaError_t launch_finalize_batched(const TileRec* recs, int T, int total_strip, int total_fin,
                                     cudaStream_t s);
 cudaError_t launch_count_active(const DevState* states, int T, int* out, cudaStream_t s);

@@ -177,6 +177,10 @@ constexpr int kDirRows = kDefaultDirRows;
 constexpr int kUpdRows = kDefaultUpdRows;
 constexpr int kSchurRows = 24;
 
+// column blocks of a W-wide image in the float4-lane launches
+__device__ __forceinline__ int vec_cols(int W) {
+    return (W + kThreads * kVec - 1) / (kThreads * kVec);
+}
 __device__ __forceinline__ void ld4(const float* __restrict__ p, float (&v)[4]) {
     const float4 t = *reinterpret_cast<const float4*>(p);
     v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
@@ -330,25 +334,29 @@ k_reweight_residual(Planes P, StencilArgs a, DevState* st, double* partials) {
 // block and z_V = r_V / (D + 1/tau) (the diagonal blocks of the preconditioner, Sec. 3.3);
 // p^T A p = sum (y_v^2 + y_h^2) / tau + D p_V^2; alpha = rho / p^T A p.
 // ------------------------------------------------------------------------------------------
-template <int ROWS>
+// ROWS > 0: rows per block fixed at compile time, 0: a.dir_rows.  UNITS (batches): the block's rows
+// are summed in units of a.dir_unit rows.
+template <int ROWS, bool UNITS>
 __device__ __forceinline__ void k_direction_pap_body(Planes P, StencilArgs a, DevState* st, double* partials, const Blk& blk) {
     if (st->done) return;
     const int H = a.H, W = a.W, ld = a.ld;
     const int j0 = (blk.bx * kThreads + threadIdx.x) * kVec;
     const int lane = threadIdx.x & 31;
-    const int R = ROWS > 0 ? ROWS : a.dir_rows;   // 0: the row count of the launch's arguments
+    const int R = ROWS > 0 ? ROWS : a.dir_rows;
     const int i0 = blk.by * R, i1 = min(i0 + R, H);
     const bool act = j0 < W;
     const float it = a.inv_tau;
     const int cur = st->pbuf, nxt = cur ^ 1;
     const bool fresh = st->p_fresh != 0;
     const float beta = fresh ? 0.f : (float)st->beta;
-    const float* __restrict__ pUo = P.pU[cur];
-    const float* __restrict__ pVvo = P.pVv[cur];
-    const float* __restrict__ pVho = P.pVh[cur];
-    float* __restrict__ pUn = P.pU[nxt];
-    float* __restrict__ pVvn = P.pVv[nxt];
-    float* __restrict__ pVhn = P.pVh[nxt];
+    // (selected, not indexed: a batch's planes come from memory, and an indexed copy of them would
+    // live in local memory)
+    const float* __restrict__ pUo = cur ? P.pU[1] : P.pU[0];
+    const float* __restrict__ pVvo = cur ? P.pVv[1] : P.pVv[0];
+    const float* __restrict__ pVho = cur ? P.pVh[1] : P.pVh[0];
+    float* __restrict__ pUn = cur ? P.pU[0] : P.pU[1];
+    float* __restrict__ pVvn = cur ? P.pVv[0] : P.pVv[1];
+    float* __restrict__ pVhn = cur ? P.pVh[0] : P.pVh[1];
     const float* __restrict__ zU = P.zU;
     const float* __restrict__ rVv = P.rVv;
     const float* __restrict__ rVh = P.rVh;
@@ -411,6 +419,8 @@ __device__ __forceinline__ void k_direction_pap_body(Planes P, StencilArgs a, De
         }
     }
     CSum acc;
+    __shared__ UnitSums<UNITS ? 1 : 0> us;
+    int unit = 0, unit_left = UNITS ? a.dir_unit : 0;
     for (int i = i0; i < i1; ++i) {
         const size_t o = (size_t)i * ld + j0;
         const bool hv = i + 1 < H;
@@ -443,9 +453,23 @@ __device__ __forceinline__ void k_direction_pap_body(Planes P, StencilArgs a, De
         }
         rcu = rnu;
         rnu = rmu;
+        if constexpr (UNITS) {
+            if (--unit_left == 0 || i + 1 == i1) {
+                const double t[1] = {acc.value()};
+                unit_done<1>(us, unit++, t);
+                acc = CSum();
+                unit_left = a.dir_unit;
+            }
+        }
     }
     double v[1] = {acc.value()}, tot[1];
-    if (grid_reduce<1>(v, partials, &st->counter, tot, blk.nblk, blk.bid) && threadIdx.x == 0) {
+    bool last;
+    if constexpr (UNITS)
+        last = grid_reduce_units<1>(us, partials, &st->counter, tot, blk, vec_cols(W),
+                                    i0 / a.dir_unit, unit, (H + a.dir_unit - 1) / a.dir_unit);
+    else
+        last = grid_reduce<1>(v, partials, &st->counter, tot, blk.nblk, blk.bid);
+    if (last && threadIdx.x == 0) {
         const double pq = tot[0];
         st->pq = pq;
         st->pbuf = nxt;
@@ -465,7 +489,7 @@ __device__ __forceinline__ void k_direction_pap_body(Planes P, StencilArgs a, De
 template <int ROWS>
 __global__ void __launch_bounds__(kThreads)
 k_direction_pap(Planes P, StencilArgs a, DevState* st, double* partials) {
-    k_direction_pap_body<ROWS>(P, a, st, partials, single_blk());
+    k_direction_pap_body<ROWS, false>(P, a, st, partials, single_blk());
 }
 
 // ------------------------------------------------------------------------------------------
@@ -473,22 +497,22 @@ k_direction_pap(Planes P, StencilArgs a, DevState* st, double* partials) {
 // eq. 'matrix-soft-constraints'), then ||r||^2, r_V^T z_V (z_V = r_V / (D + 1/tau)) and, for the
 // flexible variant, r_new^T z_old.  Stops the run when ||r|| <= cg_tol ||b|| or on cg_max.
 // ------------------------------------------------------------------------------------------
-template <int ROWS>
+template <int ROWS, bool UNITS>   // as the direction kernel's
 __device__ __forceinline__ void k_update_body(Planes P, StencilArgs a, DevState* st, double* partials, const Blk& blk) {
     if (st->done) return;
     const int H = a.H, W = a.W, ld = a.ld;
     const int j0 = (blk.bx * kThreads + threadIdx.x) * kVec;
     const int lane = threadIdx.x & 31;
-    const int R = ROWS > 0 ? ROWS : a.upd_rows;   // 0: the row count of the launch's arguments
+    const int R = ROWS > 0 ? ROWS : a.upd_rows;
     const int i0 = blk.by * R, i1 = min(i0 + R, H);
     const bool act = j0 < W;
     const float it = a.inv_tau;
     const int cur = st->pbuf;
     const float alpha = (float)st->alpha;
     const bool flex = a.flexible != 0;
-    const float* __restrict__ pU = P.pU[cur];
-    const float* __restrict__ pVv = P.pVv[cur];
-    const float* __restrict__ pVh = P.pVh[cur];
+    const float* __restrict__ pU = cur ? P.pU[1] : P.pU[0];
+    const float* __restrict__ pVv = cur ? P.pVv[1] : P.pVv[0];
+    const float* __restrict__ pVh = cur ? P.pVh[1] : P.pVh[0];
     const float* __restrict__ Dv = P.dv;
     const float* __restrict__ Dh = P.dh;
     const float* __restrict__ Zu = P.zU;
@@ -520,6 +544,8 @@ __device__ __forceinline__ void k_update_body(Planes P, StencilArgs a, DevState*
         }
     }
     CSum rr, rzv, rzo, ru2, su;
+    __shared__ UnitSums<UNITS ? 5 : 0> us;
+    int unit = 0, unit_left = UNITS ? a.upd_unit : 0;
     for (int i = i0; i < i1; ++i) {
         const size_t o = (size_t)i * ld + j0;
         const bool hv = i + 1 < H;
@@ -592,9 +618,23 @@ __device__ __forceinline__ void k_update_body(Planes P, StencilArgs a, DevState*
             cu[e] = nu[e]; cvv[e] = nvv[e]; cvh[e] = nvh[e];
             nu[e] = mu[e]; nvv[e] = mvv[e]; nvh[e] = mvh[e];
         }
+        if constexpr (UNITS) {
+            if (--unit_left == 0 || i + 1 == i1) {
+                const double t[5] = {rr.value(), rzv.value(), rzo.value(), ru2.value(), su.value()};
+                unit_done<5>(us, unit++, t);
+                rr = rzv = rzo = ru2 = su = CSum();
+                unit_left = a.upd_unit;
+            }
+        }
     }
     double v[5] = {rr.value(), rzv.value(), rzo.value(), ru2.value(), su.value()}, tot[5];
-    if (grid_reduce<5>(v, partials, &st->counter, tot, blk.nblk, blk.bid) && threadIdx.x == 0) {
+    bool last;
+    if constexpr (UNITS)
+        last = grid_reduce_units<5>(us, partials, &st->counter, tot, blk, vec_cols(W),
+                                    i0 / a.upd_unit, unit, (H + a.upd_unit - 1) / a.upd_unit);
+    else
+        last = grid_reduce<5>(v, partials, &st->counter, tot, blk.nblk, blk.bid);
+    if (last && threadIdx.x == 0) {
         const double rr_range = range_part(tot[0], tot[4], a.H, a.W);
         st->rr = rr_range;
         st->rz_v = tot[1];
@@ -612,7 +652,7 @@ __device__ __forceinline__ void k_update_body(Planes P, StencilArgs a, DevState*
 template <int ROWS>
 __global__ void __launch_bounds__(kThreads)
 k_update(Planes P, StencilArgs a, DevState* st, double* partials) {
-    k_update_body<ROWS>(P, a, st, partials, single_blk());
+    k_update_body<ROWS, false>(P, a, st, partials, single_blk());
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1023,16 +1063,15 @@ __global__ void __launch_bounds__(kThreads) kb_reweight(const TileRec* __restric
     k_reweight_residual_body<0>(r.P, r.a, r.st, r.partials, tile_blk(r, blockIdx.x, GK_RW));
 }
 
-template <int ROWS>
-__global__ void __launch_bounds__(kThreads) kb_direction(const TileRec* __restrict__ recs, int T) {
+// direction and update: each image with its own rows per block and summation unit (unit_rows)
+__global__ void __launch_bounds__(kThreads, 5) kb_direction(const TileRec* __restrict__ recs, int T) {
     const TileRec& r = recs[find_tile(recs, T, blockIdx.x, GK_DIR)];
-    k_direction_pap_body<ROWS>(r.P, r.a, r.st, r.partials, tile_blk(r, blockIdx.x, GK_DIR));
+    k_direction_pap_body<0, true>(r.P, r.a, r.st, r.partials, tile_blk(r, blockIdx.x, GK_DIR));
 }
 
-template <int ROWS>
-__global__ void __launch_bounds__(kThreads) kb_update(const TileRec* __restrict__ recs, int T) {
+__global__ void __launch_bounds__(kThreads, 4) kb_update(const TileRec* __restrict__ recs, int T) {
     const TileRec& r = recs[find_tile(recs, T, blockIdx.x, GK_UPD)];
-    k_update_body<ROWS>(r.P, r.a, r.st, r.partials, tile_blk(r, blockIdx.x, GK_UPD));
+    k_update_body<0, true>(r.P, r.a, r.st, r.partials, tile_blk(r, blockIdx.x, GK_UPD));
 }
 
 __global__ void __launch_bounds__(kThreads) kb_finalize(const TileRec* __restrict__ recs, int T) {
@@ -1483,12 +1522,7 @@ void strip_dims(int H, int W, int& gx, int& gy) {
     gy = (int)g.y;
 }
 
-void vec_dims(int H, int W, int dir_rows, int upd_rows, int& gx, int& gy_dir, int& gy_upd) {
-    dim3 g = vec_grid(H, W, dir_rows);
-    gx = (int)g.x;
-    gy_dir = (int)g.y;
-    gy_upd = (int)vec_grid(H, W, upd_rows).y;
-}
+int vec_blocks_x(int W) { return (int)vec_grid(1, W, 1).x; }
 
 cudaError_t launch_init_batched(const TileRec* recs, int T, int total, cudaStream_t s) {
     kb_init<<<total, kThreads, 0, s>>>(recs, T);
@@ -1505,27 +1539,13 @@ cudaError_t launch_reweight_batched(const TileRec* recs, int T, int total_rw, cu
     return cudaGetLastError();
 }
 
-cudaError_t launch_direction_batched(const TileRec* recs, int T, int total, int rows,
-                                     cudaStream_t s) {
-    switch (rows) {
-        case 8: kb_direction<8><<<total, kThreads, 0, s>>>(recs, T); break;
-        case 16: kb_direction<16><<<total, kThreads, 0, s>>>(recs, T); break;
-        case 24: kb_direction<24><<<total, kThreads, 0, s>>>(recs, T); break;
-        case 32: kb_direction<32><<<total, kThreads, 0, s>>>(recs, T); break;
-        default: return cudaErrorInvalidValue;
-    }
+cudaError_t launch_direction_batched(const TileRec* recs, int T, int total, cudaStream_t s) {
+    kb_direction<<<total, kThreads, 0, s>>>(recs, T);
     return cudaGetLastError();
 }
 
-cudaError_t launch_update_batched(const TileRec* recs, int T, int total, int rows,
-                                  cudaStream_t s) {
-    switch (rows) {
-        case 8: kb_update<8><<<total, kThreads, 0, s>>>(recs, T); break;
-        case 16: kb_update<16><<<total, kThreads, 0, s>>>(recs, T); break;
-        case 24: kb_update<24><<<total, kThreads, 0, s>>>(recs, T); break;
-        case 32: kb_update<32><<<total, kThreads, 0, s>>>(recs, T); break;
-        default: return cudaErrorInvalidValue;
-    }
+cudaError_t launch_update_batched(const TileRec* recs, int T, int total, cudaStream_t s) {
+    kb_update<<<total, kThreads, 0, s>>>(recs, T);
     return cudaGetLastError();
 }
 
@@ -1543,21 +1563,33 @@ cudaError_t launch_count_active(const DevState* states, int T, int* out, cudaStr
     return cudaGetLastError();
 }
 
-int wave_rows(int kernel, int H, int W, int max_rows) {
+// blocks of a float4-lane kernel the device runs at once (0: unknown)
+static long long resident_blocks(int kernel) {
     static const void* const fn[6] = {(const void*)k_direction_pap<0>, (const void*)k_update<0>,
                                       (const void*)k_reweight_residual<0>,
                                       (const void*)k_finalize_reduce<0>,
                                       (const void*)k_schur_direction<0>,
                                       (const void*)k_schur_update<0>};
-    if (kernel < 0 || kernel > 5 || H < 1 || W < 1) return 0;
+    if (kernel < 0 || kernel > 5) return 0;
     int dev = 0, sms = 0, per = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn[kernel], kThreads, 0) !=
             cudaSuccess || sms < 1 || per < 1)
         return 0;
-    const int gx = (int)vec_grid(H, W, kMinTileRows).x;
-    const long long slots = (long long)sms * per;
+    return std::min<long long>((long long)sms * per, kMaxWaveBlocks);
+}
+
+int one_wave_rows(int kernel, int H, int W) {
+    if (H < 1 || W < 1) return 0;
+    const long long strips = resident_blocks(kernel) / vec_blocks_x(W);
+    return strips < 1 ? 0 : (int)((H + strips - 1) / strips);
+}
+
+int wave_rows(int kernel, int H, int W, int max_rows) {
+    const long long slots = resident_blocks(kernel);
+    if (slots < 1 || H < 1 || W < 1) return 0;
+    const int gx = vec_blocks_x(W);
     // the fewest waves k whose row strips (k slots / gx of them) need at most max_rows rows each
     for (int k = 1; k <= 64; ++k) {
         const long long strips = k * slots / gx;
@@ -1571,6 +1603,8 @@ int wave_rows(int kernel, int H, int W, int max_rows) {
 }
 
 int aux_rows(int kernel, int H, int W) {
+    const int one = one_wave_rows(kernel, H, W);
+    if (one > 0 && one < kMinTileRows) return one;
     const int r = wave_rows(kernel, H, W, kMaxTileRows);
     return r ? r : kDefaultUpdRows;
 }
@@ -1578,7 +1612,7 @@ int aux_rows(int kernel, int H, int W) {
 int stencil_grid_blocks(int H, int W) {
     dim3 g = strip_grid(H, W), v = vec_grid(H, W, std::min({kDirRows, kUpdRows, kSchurRows,
                                                            kTileRows[0]}));
-    return (int)std::max(g.x * g.y, v.x * v.y);
+    return (int)std::max<unsigned>({g.x * g.y, v.x * v.y, (unsigned)kMaxWaveBlocks});
 }
 
 namespace {
@@ -1595,7 +1629,7 @@ cudaError_t launch_rows(int rows, int H, int W, cudaStream_t s, Args... args) {
         default:
             // any other count in range: the runtime-rows instance (the count travels in the
             // kernel's arguments)
-            if (!plan_rows_ok(rows)) return cudaErrorInvalidValue;
+            if (rows < 1 || rows > kMaxTileRows) return cudaErrorInvalidValue;
             K<0>::go(vec_grid(H, W, rows), s, args...);
             break;
     }
@@ -1658,21 +1692,21 @@ cudaError_t launch_norm_u(const Planes& P, const StencilArgs& a, DevState* st, d
 cudaError_t launch_reweight_residual(const Planes& P, const StencilArgs& a, DevState* st,
                                      double* partials, cudaStream_t s) {
     StencilArgs b = a;
-    b.rw_rows = plan_rows_ok(a.rw_rows) ? a.rw_rows : rows_or(a.upd_rows, kUpdRows);
+    b.rw_rows = a.rw_rows > 0 ? a.rw_rows : rows_or(a.upd_rows, kUpdRows);
     return launch_rows<RwK>(b.rw_rows, a.H, a.W, s, P, b, st, partials);
 }
 
 cudaError_t launch_direction_pap(const Planes& P, const StencilArgs& a, DevState* st,
                                  double* partials, cudaStream_t s) {
     StencilArgs b = a;
-    b.dir_rows = rows_or(a.dir_rows, kDirRows);
+    b.dir_rows = unit_rows(rows_or(a.dir_rows, kDirRows), a.dir_wave);
     return launch_rows<DirK>(b.dir_rows, a.H, a.W, s, P, b, st, partials);
 }
 
 cudaError_t launch_update(const Planes& P, const StencilArgs& a, DevState* st, double* partials,
                           cudaStream_t s) {
     StencilArgs b = a;
-    b.upd_rows = rows_or(a.upd_rows, kUpdRows);
+    b.upd_rows = unit_rows(rows_or(a.upd_rows, kUpdRows), a.upd_wave);
     return launch_rows<UpdK>(b.upd_rows, a.H, a.W, s, P, b, st, partials);
 }
 
@@ -1685,7 +1719,7 @@ cudaError_t launch_schur_reweight(const Planes& P, const StencilArgs& a, DevStat
 // U-only CG kernels: the plan's whole-wave row counts (a.sdir_rows, a.supd_rows), else 24 rows
 cudaError_t launch_schur_direction(const Planes& P, const StencilArgs& a, DevState* st,
                                    double* partials, cudaStream_t s) {
-    const int rows = plan_rows_ok(a.sdir_rows) ? a.sdir_rows : kSchurRows;
+    const int rows = a.sdir_rows > 0 ? a.sdir_rows : kSchurRows;
     if (rows == kSchurRows)
         k_schur_direction<kSchurRows><<<vec_grid(a.H, a.W, rows), kThreads, 0, s>>>(P, a, st,
                                                                                    partials);
@@ -1696,7 +1730,7 @@ cudaError_t launch_schur_direction(const Planes& P, const StencilArgs& a, DevSta
 
 cudaError_t launch_schur_update(const Planes& P, const StencilArgs& a, DevState* st,
                                 double* partials, cudaStream_t s) {
-    const int rows = plan_rows_ok(a.supd_rows) ? a.supd_rows : kSchurRows;
+    const int rows = a.supd_rows > 0 ? a.supd_rows : kSchurRows;
     if (rows == kSchurRows)
         k_schur_update<kSchurRows><<<vec_grid(a.H, a.W, rows), kThreads, 0, s>>>(P, a, st,
                                                                                 partials);
@@ -1713,7 +1747,7 @@ cudaError_t launch_schur_recover_v(const Planes& P, const StencilArgs& a, cudaSt
 cudaError_t launch_finalize(const Planes& P, const StencilArgs& a, DevState* st, double* partials,
                             cudaStream_t s) {
     StencilArgs b = a;
-    b.fin_rows = plan_rows_ok(a.fin_rows) ? a.fin_rows : rows_or(a.upd_rows, kUpdRows);
+    b.fin_rows = a.fin_rows > 0 ? a.fin_rows : rows_or(a.upd_rows, kUpdRows);
     cudaError_t e = launch_rows<FinK>(b.fin_rows, a.H, a.W, s, P, b, st, partials);
     if (e != cudaSuccess) return e;
     k_subtract_mean<<<strip_grid(a.H, a.W), kThreads, 0, s>>>(P.U, a.H, a.W, a.ld, st);

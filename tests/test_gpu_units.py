@@ -1,0 +1,44 @@
+"""Summation units of the direction and update kernels: a single image's blocks hold one unit, a
+batch's several, and both sum the same units in the same order."""
+import numpy as np
+import pytest
+
+import synthetic
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def irls():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2401_09961_gb300 as m
+    m.lib()
+    return m
+
+
+def cuda(a):
+    return torch.as_tensor(np.ascontiguousarray(a, dtype=np.float32)).cuda()
+
+
+# units of one row (few blocks), of several rows that do not divide the height, of the tile's own
+# rows (the last), one row only, one column block and several
+SHAPES = [(1, 700), (100, 300), (333, 513), (701, 1003), (97, 2600), (2100, 1300)]
+
+
+@pytest.mark.parametrize("tiles", [(24, 32), (8, 8)])
+def test_batch_units_equal_single_plans(irls, tiles):
+    opts = dict(tau=1e-2, delta=1e-3, outer_iters=2, cg_tol=1e-6, cg_max_iter=60,
+                precision="bf16x3", dct_form="direct")
+    data = [synthetic.config_2048(seed=900 + t, H=h, W=w) for t, (h, w) in enumerate(SHAPES)]
+    with irls.Batch(SHAPES, **opts) as b:
+        b.set_tiles(*tiles)
+        Us, st = b.unwrap([cuda(d["X"]) for d in data], [cuda(d["coherence"]) for d in data])
+    for t, (h, w) in enumerate(SHAPES):
+        with irls.Plan(h, w, **opts) as p:
+            p.set_tiles(*tiles)
+            U, s1 = p.unwrap(cuda(data[t]["X"]), cuda(data[t]["coherence"]))
+        assert torch.equal(Us[t], U), SHAPES[t]
+        assert st[t]["cg_iters"] == s1["cg_iters"] and st[t]["l1_obj"] == s1["l1_obj"], SHAPES[t]
