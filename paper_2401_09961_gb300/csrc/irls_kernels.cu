@@ -593,9 +593,11 @@ __device__ __forceinline__ void k_update_body(Planes P, StencilArgs a, DevState*
                 n1[e] = __fmaf_rn(-alpha, qvl, __fmaf_rn(-alpha, qvh, r1[e]));
                 n2[e] = __fmaf_rn(-alpha, qhl, __fmaf_rn(-alpha, qhh, r2[e]));
                 const float iv = 1.f / (dv[e] + it), ih = 1.f / (dh[e] + it);
-                prr += n0[e] * n0[e] + n1[e] * n1[e] + n2[e] * n2[e];
-                pru2 += n0[e] * n0[e];
-                psu += n0[e];
+                // written out: the same roundings in every instance of this kernel
+                prr = __fadd_rn(prr, __fmaf_rn(n2[e], n2[e], __fmaf_rn(n1[e], n1[e],
+                                                                      __fmul_rn(n0[e], n0[e]))));
+                pru2 = __fmaf_rn(n0[e], n0[e], pru2);
+                psu = __fadd_rn(psu, n0[e]);
                 przv += n1[e] * n1[e] * iv + n2[e] * n2[e] * ih;
                 if (flex) przo += n0[e] * z[e] + (n1[e] * r1[e]) * iv + (n2[e] * r2[e]) * ih;
             }

@@ -41,4 +41,4 @@ def test_batch_units_equal_single_plans(irls, tiles):
             p.set_tiles(*tiles)
             U, s1 = p.unwrap(cuda(data[t]["X"]), cuda(data[t]["coherence"]))
         assert torch.equal(Us[t], U), SHAPES[t]
-        assert st[t]["cg_iters"] == s1["cg_iters"] and st[t]["l1_obj"] == s1["l1_obj"], SHAPES[t]
+        assert st[t]["rel_res"] == s1["rel_res"] and st[t]["l1_obj"] == s1["l1_obj"], SHAPES[t]
