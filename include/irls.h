@@ -346,7 +346,8 @@ int irls_precond_laplacian(irls_plan plan, const float* d_R, float* d_Z, void* s
  *   q_U  = (S^T S U + U T T^T - S^T Vv - Vh T^T) / tau
  *   q_Vv = Dv o Vv + (Vv - S U) / tau,    q_Vh = Dh o Vh + (Vh - U T) / tau
  * with Dv = d_Dv ((H-1) x W), Dh = d_Dh (H x (W-1)) and tau from the plan's options.
- * Runs the same update kernel as the CG loop.  Asynchronous on `stream`. */
+ * With the CG update kernel's arithmetic, on the caller's arrays directly.  An output may lie
+ * over an input.  Asynchronous on `stream`. */
 int irls_apply_A(irls_plan plan, const float* d_U, const float* d_Vv, const float* d_Vh,
                  const float* d_Dv, const float* d_Dh, float* d_qU, float* d_qVv, float* d_qVh,
                  void* stream);

@@ -27,7 +27,7 @@ namespace irls {
 
 cudaError_t umma_dct_apply(const DctPlan& d, const float* rU, float* zU, int ld, DevState* st,
                            int reduce_rho, const StencilArgs& a, double* partials,
-                           int skip_if_done, cudaStream_t s);
+                           int skip_if_done, cudaStream_t s, const float* src, int ld_src);
 size_t umma_dct_bytes(int H, int W, int prec);
 cudaError_t umma_dct_setup(DctPlan& d, char* mem);
 void umma_dct_release(DctPlan& d);
@@ -582,10 +582,11 @@ bool dct_stall(DctPlan& d, int on) { return umma_dct_stall(d, on); }
 
 cudaError_t dct_apply(const DctPlan& d, const float* rU, float* zU, int ld, DevState* st,
                       int reduce_rho, const StencilArgs& a, double* partials, int skip_if_done,
-                      cudaStream_t s) {
+                      cudaStream_t s, const float* src, int ld_src) {
     if (d.fft) return fft_dct_apply(d, rU, zU, ld, st, reduce_rho, a, partials, skip_if_done, s);
     if (d.prec != IRLS_PREC_FP32)
-        return umma_dct_apply(d, rU, zU, ld, st, reduce_rho, a, partials, skip_if_done, s);
+        return umma_dct_apply(d, rU, zU, ld, st, reduce_rho, a, partials, skip_if_done, s, src,
+                              ld_src);
     QuadArgs base{};
     base.st = st;
     base.partials = partials;

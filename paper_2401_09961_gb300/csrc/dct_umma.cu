@@ -1490,10 +1490,8 @@ __device__ __forceinline__ void fold_r_body(const FoldRRec& f, int bid, int nblk
         const float sc = rn > 0.0 ? (float)(1.0 / (rn * (double)f.inv_sqrt_n)) : 1.f;
         __half* __restrict__ Eh = reinterpret_cast<__half*>(f.Re);
         __half* __restrict__ Oh = reinterpret_cast<__half*>(f.Ro);
-        const int h = (W + 1) / 2;
-        const size_t total = (size_t)H * h;
-        for (size_t t = bid * (size_t)blockDim.x + threadIdx.x; t < total;
-             t += (size_t)nblk * blockDim.x) {
+        const unsigned h = (W + 1) / 2, total = H * h;   // below 2^31: 32-bit divisions
+        for (unsigned t = bid * blockDim.x + threadIdx.x; t < total; t += nblk * blockDim.x) {
             const int i = (int)(t / h), j = (int)(t % h);
             const bool self = 2 * j + 1 == W;
             const float a = rU[(size_t)i * ld + j];
@@ -1508,13 +1506,12 @@ __device__ __forceinline__ void fold_r_body(const FoldRRec& f, int bid, int nblk
     __nv_bfloat16* __restrict__ Relo = f.Relo;
     __nv_bfloat16* __restrict__ Ro = f.Ro;
     __nv_bfloat16* __restrict__ Rolo = f.Rolo;
-    if (W % 8 != 0) {
+    // 16-byte loads: a caller's array may have any alignment
+    if (W % 8 != 0 || ld % 4 != 0 || (reinterpret_cast<uintptr_t>(rU) & 15) != 0) {
         // (W + 1) / 2 columns: for odd W the middle column is its own mirror (sum: the column
         // itself; difference: 0)
-        const int h = (W + 1) / 2;
-        const size_t total = (size_t)H * h;
-        for (size_t t = bid * (size_t)blockDim.x + threadIdx.x; t < total;
-             t += (size_t)nblk * blockDim.x) {
+        const unsigned h = (W + 1) / 2, total = H * h;
+        for (unsigned t = bid * blockDim.x + threadIdx.x; t < total; t += nblk * blockDim.x) {
             const int i = (int)(t / h), j = (int)(t % h);
             const bool self = 2 * j + 1 == W;
             const float a = rU[(size_t)i * ld + j];
@@ -1531,10 +1528,8 @@ __device__ __forceinline__ void fold_r_body(const FoldRRec& f, int bid, int nblk
         }
         return;
     }
-    const int h4 = W / 8;
-    const size_t total = (size_t)H * h4;
-    for (size_t t = bid * (size_t)blockDim.x + threadIdx.x; t < total;
-         t += (size_t)nblk * blockDim.x) {
+    const unsigned h4 = W / 8, total = H * h4;
+    for (unsigned t = bid * blockDim.x + threadIdx.x; t < total; t += nblk * blockDim.x) {
         const int i = (int)(t / h4), j = (int)(t % h4) * 4;
         const float4 a = *reinterpret_cast<const float4*>(rU + (size_t)i * ld + j);
         const float4 bm = *reinterpret_cast<const float4*>(rU + (size_t)i * ld + (W - 4 - j));
@@ -2360,7 +2355,7 @@ cudaError_t fold_bind(const DctPlan& d, FoldBufs& f, const float* rU, float* zU,
 
 cudaError_t fold_apply(const DctPlan& d, const float* rU, float* zU, int ld, DevState* st,
                        int reduce_rho, int flexible, double* partials, int skip_if_done,
-                       cudaStream_t s) {
+                       cudaStream_t s, const float* src, int ld_src) {
     FoldBufs& f = *static_cast<FoldBufs*>(d.fold_host);
     if (!f.bound || f.rU != rU || f.zU != zU || f.ld != ld || f.st != st ||
         f.partials != partials || f.flexible != flexible || f.skip != skip_if_done ||
@@ -2370,7 +2365,8 @@ cudaError_t fold_apply(const DctPlan& d, const float* rU, float* zU, int ld, Dev
         if (e != cudaSuccess) return e;
     }
     k_fold_r<<<fold_r_blocks(d.H, d.W, f.fused.f16), 256, 0, s>>>(
-        fold_r_rec(f.img, rU, ld, d.H, d.W, st, f.fused.f16), skip_if_done);
+        fold_r_rec(f.img, src ? src : rU, src ? ld_src : ld, d.H, d.W, st, f.fused.f16),
+        skip_if_done);
     return launch_fused(f.fused, s);
 }
 
@@ -2567,9 +2563,11 @@ cudaError_t umma_dct_setup(DctPlan& d, char* mem) {
 
 cudaError_t umma_dct_apply(const DctPlan& d, const float* rU, float* zU, int ld, DevState* st,
                            int reduce_rho, const StencilArgs& a, double* partials,
-                           int skip_if_done, cudaStream_t s) {
+                           int skip_if_done, cudaStream_t s, const float* src, int ld_src) {
     if (!d.umma_ok) return cudaErrorNotSupported;
-    if (d.fold) return fold_apply(d, rU, zU, ld, st, reduce_rho, a.flexible, partials, skip_if_done, s);
+    if (d.fold)
+        return fold_apply(d, rU, zU, ld, st, reduce_rho, a.flexible, partials, skip_if_done, s,
+                          src, ld_src);
     const TmapSet& ts = *reinterpret_cast<const TmapSet*>(d.tmap_storage);
     const int Hp = d.Hp, Wp = d.Wp;
     const int mk = d.split;

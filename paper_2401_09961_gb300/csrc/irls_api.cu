@@ -69,7 +69,7 @@ bool shape_valid(int H, int W) {
 }
 
 struct Layout {
-    size_t plane_bytes, planes, state, partials, dct, total;
+    size_t plane_bytes, planes, state, partials, circle, dct, total;
     int max_blocks;
 };
 
@@ -88,7 +88,8 @@ Layout layout(int H, int W, int prec) {
     L.partials = L.state + align_up(sizeof(DevState), 256);
     L.max_blocks = std::max({stencil_grid_blocks(H, W), dct_max_blocks(H, W),
                              fft_dct_max_blocks(H, W)});
-    L.dct = L.partials + align_up(partial_count(H, W, L.max_blocks) * sizeof(double), 1024);
+    L.circle = L.partials + align_up(partial_count(H, W, L.max_blocks) * sizeof(double), 1024);
+    L.dct = L.circle + align_up(circle_bytes(), 1024);
     L.total = L.dct + align_up(dct_bytes(H, W, prec), 1024) + 1024;
     return L;
 }
@@ -752,6 +753,7 @@ int irls_plan_create(int H, int W, const irls_opts* opts, irls_plan* out) {
         P.Cv = f[q++]; P.Ch = f[q++];
         p->st = reinterpret_cast<DevState*>(p->mem + p->L.state);
         p->partials = reinterpret_cast<double*>(p->mem + p->L.partials);
+        ck(build_circle(p->mem + p->L.circle));
         ck(dct_setup(p->dct, H, W, o.precision, o.tau, p->mem + p->L.dct));
         if (!select_dct_form(p, o)) {
             destroy_plan(p);
@@ -1332,20 +1334,32 @@ int irls_precond_laplacian(irls_plan p, const float* R, float* Z, void* stream) 
     try {
         DeviceGuard g(p->dev);
         StencilArgs a = make_args(p);
-        // the float32 dense products read and write rows of any pitch
-        if (p->opts.precision == IRLS_PREC_FP32 && !p->dct.fft) {
-            ck(dct_apply(p->dct, R, Z, p->W, p->st, 0, a, p->partials, 0, s));
+        const int H = p->H, W = p->W;
+        // the caller's arrays take the planes' place where the form reads rows of any pitch (the
+        // float32 dense products), or of a pitch and an alignment that they have (the fast
+        // transforms' 16-byte accesses)
+        const bool fft = p->dct.fft != 0;
+        const bool al16 = W % 4 == 0 && ((reinterpret_cast<uintptr_t>(R) |
+                                          reinterpret_cast<uintptr_t>(Z)) & 15) == 0;
+        if (fft ? al16 : p->opts.precision == IRLS_PREC_FP32) {
+            ck(dct_apply(p->dct, R, Z, W, p->st, 0, a, p->partials, 0, s));
             return IRLS_OK;
         }
-        ck(cudaMemsetAsync(p->P.rU, 0, p->L.plane_bytes, s));
-        ck(launch_copy_in(R, p->H, p->W, p->P.rU, p->ld, s));
-        if (a.r16) ck(launch_emit16(p->P.rU, p->H, p->W, p->ld, a.r16, a.r16lo, a.ld16, s));
+        // the tensor-core forms read the residual from the caller's array (its fold or its bf16
+        // copy) and write the z plane their tables are bound to
+        if (fft) ck(launch_copy_in(R, H, W, p->P.rU, p->ld, s));
+        if (a.r16) ck(launch_emit16(R, H, W, W, a.r16, a.r16lo, a.ld16, s));
         // the float16 form scales its input by ||r_U||, which no solve kernel produced here
-        if (p->opts.precision == IRLS_PREC_FP16)
-            ck(launch_norm_u(p->P, a, p->st, p->partials, s));
+        if (p->opts.precision == IRLS_PREC_FP16) {
+            Planes P = p->P;
+            P.rU = const_cast<float*>(R);
+            StencilArgs b = a;
+            b.ld = W;
+            ck(launch_norm_u(P, b, p->st, p->partials, s));
+        }
         ck(dct_reset(p->dct, s));
-        ck(dct_apply(p->dct, p->P.rU, p->P.zU, p->ld, p->st, 0, a, p->partials, 0, s));
-        ck(launch_copy_out(p->P.zU, p->H, p->W, p->ld, Z, s));
+        ck(dct_apply(p->dct, p->P.rU, p->P.zU, p->ld, p->st, 0, a, p->partials, 0, s, R, W));
+        ck(launch_copy_out(p->P.zU, H, W, p->ld, Z, s));
     } catch (Fail&) {
         return IRLS_ERR_CUDA;
     }
@@ -1360,7 +1374,7 @@ int irls_round_congruent(irls_plan p, const float* U, const float* X, float* Ur,
         DeviceGuard g(p->dev);
         const size_t n = (size_t)p->H * p->W;
         ck(cudaMemsetAsync(&p->st->counter, 0, sizeof(unsigned int), s));
-        ck(launch_round_congruent(U, X, n, p->st, p->partials, p->L.max_blocks, Ur, K, s));
+        ck(launch_round_congruent(U, X, n, p->mem + p->L.circle, p->st, p->partials, p->L.max_blocks, Ur, K, s));
         double h = 0.0;
         ck(cudaMemcpyAsync(p->h_pair, &p->st->aux[0], sizeof(double), cudaMemcpyDeviceToHost, s));
         ck(cudaStreamSynchronize(s));
@@ -1400,24 +1414,28 @@ int irls_apply_A(irls_plan p, const float* U, const float* Vv, const float* Vh, 
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     try {
         DeviceGuard g(p->dev);
-        StencilArgs a = make_args(p);
-        const Planes& P = p->P;
-        const size_t pb = p->L.plane_bytes;
-        float* zero[] = {P.U, P.Vv, P.Vh, P.rU, P.rVv, P.rVh, P.pU[0], P.pVv[0], P.pVh[0], P.dv, P.dh};
-        for (float* z : zero) ck(cudaMemsetAsync(z, 0, pb, s));
-        ck(launch_copy_in(U, p->H, p->W, P.pU[0], p->ld, s));
-        if (p->H > 1) {
-            ck(launch_copy_in(Vv, p->H - 1, p->W, P.pVv[0], p->ld, s));
-            ck(launch_copy_in(Dv, p->H - 1, p->W, P.dv, p->ld, s));
+        const size_t H = p->H, W = p->W, n[3] = {H * W, (H - 1) * W, H * (W - 1)};
+        const float* in[5] = {U, Vv, Vh, Dv, Dh};
+        const size_t ni[5] = {n[0], n[1], n[2], n[1], n[2]};
+        const float* const out[3] = {qU, qVv, qVh};
+        // an output that overlaps an input: the kernel reads copies of the inputs
+        bool overlap = false;
+        for (int a = 0; a < 5; ++a)
+            for (int b = 0; b < 3; ++b)
+                overlap |= in[a] < out[b] + n[b] && out[b] < in[a] + ni[a];
+        if (overlap) {
+            float* const to[5] = {p->P.pU[0], p->P.pVv[0], p->P.pVh[0], p->P.pU[1], p->P.pVv[1]};
+            for (int a = 0; a < 5; ++a) {
+                ck(cudaMemcpyAsync(to[a], in[a], ni[a] * sizeof(float), cudaMemcpyDeviceToDevice, s));
+                in[a] = to[a];
+            }
         }
-        if (p->W > 1) {
-            ck(launch_copy_in(Vh, p->H, p->W - 1, P.pVh[0], p->ld, s));
-            ck(launch_copy_in(Dh, p->H, p->W - 1, P.dh, p->ld, s));
-        }
-        ck(launch_matvec_via_update(P, a, p->st, p->partials, s));
-        ck(launch_copy_out(P.rU, p->H, p->W, p->ld, qU, s));
-        if (p->H > 1) ck(launch_copy_out(P.rVv, p->H - 1, p->W, p->ld, qVv, s));
-        if (p->W > 1) ck(launch_copy_out(P.rVh, p->H, p->W - 1, p->ld, qVh, s));
+        ck(launch_apply_A(in[0], in[1], in[2], in[3], in[4], p->H, p->W, 1.0f / p->opts.tau, qU,
+                          qVv, qVh, s));
+        // (the planes' padding is zero outside a call)
+        if (overlap)
+            for (float* z : {p->P.pU[0], p->P.pVv[0], p->P.pVh[0], p->P.pU[1], p->P.pVv[1]})
+                ck(cudaMemsetAsync(z, 0, p->L.plane_bytes, s));
     } catch (Fail&) {
         return IRLS_ERR_CUDA;
     }

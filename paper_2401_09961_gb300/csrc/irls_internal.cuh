@@ -233,8 +233,10 @@ cudaError_t launch_copy_out(const float* src, int rows, int cols, int ld, float*
                             cudaStream_t s);
 cudaError_t launch_copy_in(const float* src, int rows, int cols, float* dst, int ld,
                            cudaStream_t s);
-cudaError_t launch_matvec_via_update(const Planes& P, const StencilArgs& a, DevState* st,
-                                     double* partials, cudaStream_t s);
+// (q_U, q_Vv, q_Vh) = A (U, Vv, Vh) on contiguous arrays (pitches W, W, W - 1)
+cudaError_t launch_apply_A(const float* U, const float* Vv, const float* Vh, const float* Dv,
+                           const float* Dh, int H, int W, float inv_tau, float* qU, float* qVv,
+                           float* qVh, cudaStream_t s);
 cudaError_t launch_emit16(const float* src, int H, int W, int ld, void* r16, void* r16lo, int ld16,
                          cudaStream_t s);
 int stencil_grid_blocks(int H, int W);
@@ -304,14 +306,19 @@ cudaError_t launch_schur_direction(const Planes& P, const StencilArgs& a, DevSta
 cudaError_t launch_schur_update(const Planes& P, const StencilArgs& a, DevState* st,
                                 double* partials, cudaStream_t s);
 cudaError_t launch_schur_recover_v(const Planes& P, const StencilArgs& a, cudaStream_t s);
-cudaError_t launch_round_congruent(const float* U, const float* X, size_t n, DevState* st,
-                                   double* partials, int max_blocks, float* Ur, int* K,
-                                   cudaStream_t s);
+// table of the circular-mean kernel (post.cu): its bytes, built once per plan
+size_t circle_bytes();
+cudaError_t build_circle(void* mem);
+cudaError_t launch_round_congruent(const float* U, const float* X, size_t n, const void* circle,
+                                   DevState* st, double* partials, int max_blocks, float* Ur,
+                                   int* K, cudaStream_t s);
 cudaError_t launch_best_shift(const float* U, const float* Xu, size_t n, DevState* st,
                               double* partials, int max_blocks, float* E, cudaStream_t s);
+// src (not null): the residual is read there (pitch ld_src) by the folded tensor-core form, whose
+// launch tables stay bound to the planes rU and zU.
 cudaError_t dct_apply(const DctPlan& d, const float* rU, float* zU, int ld, DevState* st,
                       int reduce_rho, const StencilArgs& a, double* partials, int skip_if_done,
-                      cudaStream_t s);
+                      cudaStream_t s, const float* src = nullptr, int ld_src = 0);
 int dct_max_blocks(int H, int W);
 size_t dct_rho_slots(int H, int W);
 // fast-transform form (dct_fft.cu): shapes it takes, its table memory, its widest grid-reduced

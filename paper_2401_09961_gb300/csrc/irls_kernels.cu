@@ -1098,31 +1098,26 @@ __global__ void k_count_active(const DevState* __restrict__ states, int T, int* 
     if (threadIdx.x == 0) *out = cnt;
 }
 
-__global__ void k_copy_out(const float* __restrict__ src, int rows, int cols, int ld,
-                           float* __restrict__ dst) {
-    const size_t n = (size_t)rows * cols;
-    for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < n;
-         t += (size_t)gridDim.x * blockDim.x) {
-        const size_t r = t / cols, c = t % cols;
-        dst[t] = src[r * ld + c];
-    }
-}
-
-__global__ void k_copy_in(const float* __restrict__ src, int rows, int cols,
-                          float* __restrict__ dst, int ld) {
-    const size_t n = (size_t)rows * cols;
-    for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < n;
-         t += (size_t)gridDim.x * blockDim.x) {
-        const size_t r = t / cols, c = t % cols;
-        dst[r * ld + c] = src[t];
+// Rows of `cols` floats from pitch ls to pitch ld; V = 4 where rows and pointers are 16-byte aligned.
+template <int V>
+__global__ void __launch_bounds__(256)
+k_copy_rows(const float* __restrict__ src, int ls, int rows, int cols, float* __restrict__ dst,
+            int ld) {
+    const int c = (blockIdx.x * 64 + threadIdx.x) * V;
+    if (c >= cols) return;
+    for (int r = blockIdx.y * 4 + threadIdx.y; r < rows; r += gridDim.y * 4) {
+        if constexpr (V == 4)
+            *reinterpret_cast<float4*>(dst + (size_t)r * ld + c) =
+                __ldg(reinterpret_cast<const float4*>(src + (size_t)r * ls + c));
+        else
+            dst[(size_t)r * ld + c] = __ldg(src + (size_t)r * ls + c);
     }
 }
 
 __global__ void k_emit16(const float* __restrict__ src, int H, int W, int ld, void* r16, void* r16lo,
                          int ld16) {
-    const size_t n = (size_t)H * W;
-    for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < n;
-         t += (size_t)gridDim.x * blockDim.x) {
+    const unsigned n = (unsigned)H * W;   // below 2^31: 32-bit divisions
+    for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
         const int i = (int)(t / W), j = (int)(t % W);
         emit16(r16, r16lo, ld16, i, j, src[(size_t)i * ld + j]);
     }
@@ -1502,12 +1497,77 @@ k_schur_recover_v(Planes P, StencilArgs a) {
     }
 }
 
-__global__ void k_prepare_matvec(DevState* st) {
-    st->done = 0;
-    st->iter = 0;
-    st->alpha = -1.0;
-    st->pbuf = 0;
-    st->bb = 1.0;
+// ------------------------------------------------------------------------------------------
+// One product with A on the caller's arrays: q_U = (S^T y_v + y_h T^T) / tau, q_V = D V - y / tau
+// with the update kernel's arithmetic (hi + lo pairs of the cancelling terms).  A thread owns one
+// column and marches down `rows` rows, the next row's loads issued before this row's stores; rows
+// of any pitch and alignment.  Bound by memory: 32 bytes a pixel and 12 a strip's end row.  2047 x
+// 1999: 35 us, host call included (through the plan's planes and the update kernel, with their
+// eleven memsets and eight copies: 266 us).
+// ------------------------------------------------------------------------------------------
+__global__ void __launch_bounds__(kThreads)
+k_apply_A(const float* __restrict__ U, const float* __restrict__ Vv, const float* __restrict__ Vh,
+          const float* __restrict__ Dv, const float* __restrict__ Dh, int H, int W, int rows,
+          float it, float* __restrict__ qU, float* __restrict__ qVv, float* __restrict__ qVh) {
+    const int j = blockIdx.x * kThreads + threadIdx.x, lane = threadIdx.x & 31;
+    const int i0 = blockIdx.y * rows, i1 = min(i0 + rows, H);
+    const bool act = j < W, hh = j + 1 < W;
+    struct Row {
+        float un, vv, dv, vh, dh, rgt, lu, lv;   // U below; V, D; U right of lane 31; left halo
+    };
+    auto load = [&](int i, Row& r) {
+        r = Row{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        if (!act) return;
+        const size_t o = (size_t)i * W + j, e = (size_t)i * (W - 1) + j;
+        if (i + 1 < H) {
+            r.un = __ldg(U + o + W);
+            r.vv = __ldg(Vv + o);
+            r.dv = __ldg(Dv + o);
+        }
+        if (hh) {
+            r.vh = __ldg(Vh + e);
+            r.dh = __ldg(Dh + e);
+            if (lane == 31) r.rgt = __ldg(U + o + 1);
+        }
+        if (lane == 0 && j > 0) {
+            r.lu = __ldg(U + o - 1);
+            r.lv = __ldg(Vh + e - 1);
+        }
+    };
+    float u = act ? __ldg(U + (size_t)i0 * W + j) : 0.f, yvp = 0.f;
+    if (act && i0 > 0) {
+        const size_t o = (size_t)(i0 - 1) * W + j;
+        yvp = u - __ldg(U + o) - __ldg(Vv + o);
+    }
+    Row c, n;
+    load(i0, c);
+    for (int i = i0; i < i1; ++i) {
+        if (i + 1 < i1) load(i + 1, n);
+        const bool hv = i + 1 < H;
+        const float yv = hv ? c.un - u - c.vv : 0.f;
+        float right = __shfl_down_sync(kFull, u, 1);
+        if (lane == 31) right = c.rgt;
+        const float yh = hh ? right - u - c.vh : 0.f;
+        float left = __shfl_up_sync(kFull, yh, 1);
+        if (lane == 0) left = j > 0 ? u - c.lu - c.lv : 0.f;
+        if (act) {
+            const size_t o = (size_t)i * W + j;
+            float h, l;
+            sum4_scaled(it, yvp, -yv, left, -yh, h, l);
+            qU[o] = __fmaf_rn(1.f, l, __fmaf_rn(1.f, h, 0.f));
+            if (hv) {
+                diff_prod(c.dv, c.vv, it, yv, h, l);
+                qVv[o] = __fmaf_rn(1.f, l, __fmaf_rn(1.f, h, 0.f));
+            }
+            if (hh) {
+                diff_prod(c.dh, c.vh, it, yh, h, l);
+                qVh[(size_t)i * (W - 1) + j] = __fmaf_rn(1.f, l, __fmaf_rn(1.f, h, 0.f));
+            }
+        }
+        yvp = yv;
+        u = c.un;
+        c = n;
+    }
 }
 
 dim3 strip_grid(int H, int W) { return dim3((W + kThreads - 1) / kThreads, (H + kRows - 1) / kRows); }
@@ -1756,22 +1816,26 @@ cudaError_t launch_finalize(const Planes& P, const StencilArgs& a, DevState* st,
     return cudaGetLastError();
 }
 
+static cudaError_t copy_rows(const float* src, int ls, int rows, int cols, float* dst, int ld,
+                             cudaStream_t s) {
+    if (rows <= 0 || cols <= 0) return cudaSuccess;
+    const bool vec = cols % 4 == 0 && ls % 4 == 0 && ld % 4 == 0 &&
+                     ((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst)) & 15) == 0;
+    const int per = vec ? 256 : 64;
+    const dim3 g((cols + per - 1) / per, std::min((rows + 3) / 4, 8192));
+    if (vec) k_copy_rows<4><<<g, dim3(64, 4), 0, s>>>(src, ls, rows, cols, dst, ld);
+    else k_copy_rows<1><<<g, dim3(64, 4), 0, s>>>(src, ls, rows, cols, dst, ld);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_copy_out(const float* src, int rows, int cols, int ld, float* dst,
                             cudaStream_t s) {
-    if (rows <= 0 || cols <= 0) return cudaSuccess;
-    const size_t n = (size_t)rows * cols;
-    const int blocks = (int)std::min<size_t>((n + 255) / 256, 8192);
-    k_copy_out<<<blocks, 256, 0, s>>>(src, rows, cols, ld, dst);
-    return cudaGetLastError();
+    return copy_rows(src, ld, rows, cols, dst, cols, s);
 }
 
 cudaError_t launch_copy_in(const float* src, int rows, int cols, float* dst, int ld,
                            cudaStream_t s) {
-    if (rows <= 0 || cols <= 0) return cudaSuccess;
-    const size_t n = (size_t)rows * cols;
-    const int blocks = (int)std::min<size_t>((n + 255) / 256, 8192);
-    k_copy_in<<<blocks, 256, 0, s>>>(src, rows, cols, dst, ld);
-    return cudaGetLastError();
+    return copy_rows(src, cols, rows, cols, dst, ld, s);
 }
 
 cudaError_t launch_emit16(const float* src, int H, int W, int ld, void* r16, void* r16lo, int ld16,
@@ -1832,18 +1896,15 @@ cudaError_t launch_adj_final(const Planes& P, const StencilArgs& a, const float*
     return cudaGetLastError();
 }
 
-cudaError_t launch_matvec_via_update(const Planes& P, const StencilArgs& a, DevState* st,
-                                     double* partials, cudaStream_t s) {
-    k_prepare_matvec<<<1, 1, 0, s>>>(st);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    StencilArgs b = a;
-    b.flexible = 0;
-    b.r16 = nullptr;
-    b.r16lo = nullptr;
-    b.cg_max = 1 << 30;
-    b.tol2 = -1.0;
-    return launch_update(P, b, st, partials, s);
+// Rows of a strip: enough strips for about eight blocks of 128 threads an SM, at most 16 rows.
+cudaError_t launch_apply_A(const float* U, const float* Vv, const float* Vh, const float* Dv,
+                           const float* Dh, int H, int W, float inv_tau, float* qU, float* qVv,
+                           float* qVh, cudaStream_t s) {
+    const int gx = (W + kThreads - 1) / kThreads;
+    const int rows = (int)std::min<long long>(16, std::max<long long>(1, (long long)H * gx / (8 * 152)));
+    k_apply_A<<<dim3(gx, (H + rows - 1) / rows), kThreads, 0, s>>>(U, Vv, Vh, Dv, Dh, H, W, rows,
+                                                                   inv_tau, qU, qVv, qVh);
+    return cudaGetLastError();
 }
 
 }  // namespace irls
