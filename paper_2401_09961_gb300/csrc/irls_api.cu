@@ -3,9 +3,9 @@
 // A plan owns one device allocation that is carved into the image planes, the device-resident
 // PCG state, the reduction scratch and the DCT bases.  A solve runs Alg. 1 of arXiv 2401.09961:
 // per outer step one reweighting/residual pass, then PCG iterations (Alg. 2) whose scalars
-// (alpha, beta, rho, the stopping flag) stay on the device.  The host only issues kernels in
-// chunks and polls the device stopping flag through pinned memory, one chunk behind, so the GPU
-// never idles waiting for the host.
+// (alpha, beta, rho, the stopping flag) stay on the device.  The host issues iterations at most
+// kAhead ahead of the one the device last reported complete (a word in pinned memory), so the GPU
+// neither idles waiting for the host nor runs through many launches after the stop.
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -31,7 +31,8 @@ void set_last_cuda_error(int code) { g_last_cuda = code; }
 namespace {
 
 constexpr int kPlanes = 21;
-constexpr int kChunk = 8;
+constexpr int kChunk = 8;   // batches: CG iterations of one graph
+constexpr int kAhead = 4;   // single images: CG iterations issued ahead of the device's report
 
 struct Fail {};
 
@@ -176,13 +177,14 @@ struct irls_plan_s {
     DctPlan dct{};
     int* h_flag = nullptr;     // pinned, 2 slots
     double* h_pair = nullptr;  // pinned, 2 doubles: H_delta values read by the Sec. 4.3 rule
+    unsigned long long* h_prog = nullptr;   // pinned: the update kernels' progress reports
+    unsigned epoch = 0;                     // CG runs issued
     std::vector<int> caps;     // cap of each inner solve of the last run
     int schedule_stop = 0;
     int dir_rows = 0, upd_rows = 0;   // stencil tile shapes (0: the defaults)
     int rw_rows = 0, fin_rows = 0;    // reweighting and finalize rows (aux_rows of H, W)
     int sdir_rows = 0, supd_rows = 0; // U-only direction and update rows (whole waves)
     int dir_wave = 0, upd_wave = 0;   // one-wave rows of the direction and update kernels
-    cudaEvent_t ev[2] = {nullptr, nullptr};
     Profiler prof;
 };
 
@@ -267,8 +269,7 @@ void destroy_plan(irls_plan_s* p) {
     if (p->mem) cudaFree(p->mem);
     if (p->h_flag) cudaFreeHost(p->h_flag);
     if (p->h_pair) cudaFreeHost(p->h_pair);
-    for (auto& e : p->ev)
-        if (e) cudaEventDestroy(e);
+    if (p->h_prog) cudaFreeHost(p->h_prog);
     cudaSetDevice(cur);
     delete p;
 }
@@ -315,43 +316,55 @@ int fetch_stats(irls_plan_s* p, cudaStream_t s, irls_stats* stats) {
     return p->h_flag[0];
 }
 
-// PCG iterations (Alg. 2) after the first preconditioner application of a run: issued in chunks,
-// the device stopping flag polled one chunk behind.
-void run_cg(irls_plan_s* p, const StencilArgs& a, DevState* st, cudaStream_t s,
+// Waits until the device is at most kAhead iterations behind the `issued` ones of run `epoch`;
+// true when the run has stopped.
+bool run_stopped(irls_plan_s* p, unsigned epoch, int issued, cudaStream_t s) {
+    const volatile unsigned long long* w = p->h_prog;
+    for (unsigned spin = 1;; ++spin) {
+        const unsigned long long v = *w;
+        const bool ours = (unsigned)(v >> 32) == epoch;
+        if (ours && (v >> 31 & 1)) return true;
+        if (issued - (ours ? (int)(v & 0x7fffffffu) : 0) <= kAhead) return false;
+        if (spin % 1024 == 0) {
+            // nothing left in flight: an error, or a run that the report does not cover
+            const cudaError_t e = cudaStreamQuery(s);
+            if (e == cudaErrorNotReady) continue;
+            ck(e);
+            if (*w != v) continue;
+            ck(cudaMemcpyAsync(&p->h_flag[0], &p->st->done, sizeof(int), cudaMemcpyDeviceToHost, s));
+            ck(cudaStreamSynchronize(s));
+            return p->h_flag[0] != 0;
+        }
+    }
+}
+
+// PCG iterations (Alg. 2) after the first preconditioner application of a run.  (Chunks of eight
+// iterations, polled one chunk behind by a copied flag, ran 8 to 16 empty iterations after every
+// stop: at 256^2 with ten outer steps, half of the launches.)
+void run_cg(irls_plan_s* p, StencilArgs a, DevState* st, cudaStream_t s,
             bool schur_system = false) {
     Profiler& pf = p->prof;
     cudaEvent_t t0;
-    int issued = 0, slot = 0;
-    bool pending = false;
-    size_t mark[2] = {0, 0};
-    while (issued < a.cg_max) {
-        const int n = std::min(kChunk, a.cg_max - issued);
-        const bool schur = schur_system || p->opts.system == IRLS_SYS_SCHUR;
-        for (int c = 0; c < n; ++c) {
-            t0 = pf.begin(s);
-            if (schur) ck(launch_schur_direction(p->P, a, st, p->partials, s));
-            else ck(launch_direction_pap(p->P, a, st, p->partials, s));
-            pf.end(PC_DIRECTION, t0, s);
-            t0 = pf.begin(s);
-            if (schur) ck(launch_schur_update(p->P, a, st, p->partials, s));
-            else ck(launch_update(p->P, a, st, p->partials, s));
-            pf.end(PC_UPDATE, t0, s);
-            t0 = pf.begin(s);
-            ck(dct_apply(p->dct, p->P.rU, p->P.zU, p->ld, st, 1, a, p->partials, 1, s));
-            pf.end(PC_DCT, t0, s);
-        }
-        issued += n;
-        ck(cudaMemcpyAsync(&p->h_flag[slot], &st->done, sizeof(int), cudaMemcpyDeviceToHost, s));
-        ck(cudaEventRecord(p->ev[slot], s));
-        mark[slot] = pf.pend.size();
-        if (pending) {
-            ck(cudaEventSynchronize(p->ev[slot ^ 1]));
-            pf.drain(mark[slot ^ 1]);
-            mark[slot] -= std::min(mark[slot], mark[slot ^ 1]);
-            if (p->h_flag[slot ^ 1]) break;
-        }
-        pending = true;
-        slot ^= 1;
+    const bool schur = schur_system || p->opts.system == IRLS_SYS_SCHUR;
+    a.progress = p->h_prog;
+    a.epoch = ++p->epoch;
+    for (int issued = 0; issued < a.cg_max;) {
+        t0 = pf.begin(s);
+        if (schur) ck(launch_schur_direction(p->P, a, st, p->partials, s));
+        else ck(launch_direction_pap(p->P, a, st, p->partials, s));
+        pf.end(PC_DIRECTION, t0, s);
+        t0 = pf.begin(s);
+        if (schur) ck(launch_schur_update(p->P, a, st, p->partials, s));
+        else ck(launch_update(p->P, a, st, p->partials, s));
+        pf.end(PC_UPDATE, t0, s);
+        t0 = pf.begin(s);
+        ck(dct_apply(p->dct, p->P.rU, p->P.zU, p->ld, st, 1, a, p->partials, 1, s));
+        pf.end(PC_DCT, t0, s);
+        if (run_stopped(p, a.epoch, ++issued, s)) break;
+    }
+    if (pf.on) {
+        ck(cudaStreamSynchronize(s));
+        pf.drain(pf.pend.size());
     }
 }
 
@@ -761,7 +774,8 @@ int irls_plan_create(int H, int W, const irls_opts* opts, irls_plan* out) {
         }
         ck(cudaHostAlloc(&p->h_flag, 2 * sizeof(int), cudaHostAllocDefault));
         ck(cudaHostAlloc(&p->h_pair, 2 * sizeof(double), cudaHostAllocDefault));
-        for (auto& ev : p->ev) ck(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+        ck(cudaHostAlloc(&p->h_prog, sizeof(unsigned long long), cudaHostAllocMapped));
+        *p->h_prog = 0;
         ck(cudaDeviceSynchronize());
     } catch (Fail&) {
         destroy_plan(p);

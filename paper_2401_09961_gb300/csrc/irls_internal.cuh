@@ -119,6 +119,10 @@ struct StencilArgs {
     // image's blocks hold one unit (see unit_rows)
     int dir_wave, upd_wave;
     int dir_unit, upd_unit;     // batches: rows of a summation unit (dir_rows, upd_rows: of a block)
+    // single-image CG runs: where the update kernels report to the host (pinned memory; null: no
+    // report), and the run's number: epoch << 32 | stopped << 31 | iterations completed
+    unsigned long long* progress;
+    unsigned epoch;
 };
 
 // Rows of a summation unit for a tile of `rows` rows and a one-wave count of `wave` rows, and the

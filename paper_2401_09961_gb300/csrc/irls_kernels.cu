@@ -171,6 +171,16 @@ __device__ __forceinline__ void emit16(void* r16, void* r16lo, int ld16, int i, 
 // values stay zero) and only the edge masks hh[] exclude the edges that do not exist.
 // ------------------------------------------------------------------------------------------
 constexpr int kVec = 4;
+// One thread's report of the CG run's state to the host, which issues iterations a few ahead of it
+// (a posted write: nothing waits for it).
+__device__ __forceinline__ void report_progress(const StencilArgs& a, int iter, int done) {
+    if (a.progress != nullptr)
+        *(volatile unsigned long long*)a.progress =
+            ((unsigned long long)a.epoch << 32) | (done ? 1ull << 31 : 0ull) | (unsigned)iter;
+}
+__device__ __forceinline__ bool first_thread() {
+    return (blockIdx.x | blockIdx.y | threadIdx.x) == 0;
+}
 // rows per block of the float4-lane kernels, measured at 4096 x 4096 (16, 24 and 32 tried):
 // direction 24, update 32; the U-only kernels 24
 constexpr int kDirRows = kDefaultDirRows;
@@ -499,7 +509,10 @@ k_direction_pap(Planes P, StencilArgs a, DevState* st, double* partials) {
 // ------------------------------------------------------------------------------------------
 template <int ROWS, bool UNITS>   // as the direction kernel's
 __device__ __forceinline__ void k_update_body(Planes P, StencilArgs a, DevState* st, double* partials, const Blk& blk) {
-    if (st->done) return;
+    if (st->done) {
+        if (!UNITS && first_thread()) report_progress(a, st->iter, 1);
+        return;
+    }
     const int H = a.H, W = a.W, ld = a.ld;
     const int j0 = (blk.bx * kThreads + threadIdx.x) * kVec;
     const int lane = threadIdx.x & 31;
@@ -646,8 +659,10 @@ __device__ __forceinline__ void k_update_body(Planes P, StencilArgs a, DevState*
         st->iter = itn;
         const double rel = st->bb > 0.0 ? sqrt(rr_range / st->bb) : 0.0;
         st->rel = rel;
-        if (rel * rel <= a.tol2 || itn >= a.cg_max || !isfinite(rel)) st->done = 1;
+        const bool stop = rel * rel <= a.tol2 || itn >= a.cg_max || !isfinite(rel);
+        if (stop) st->done = 1;
         if (!isfinite(rel)) st->status |= ST_NONFINITE;
+        if (!UNITS) report_progress(a, itn, stop);
     }
 }
 
@@ -1357,7 +1372,10 @@ template <int ROWS>
 __global__ void __launch_bounds__(kThreads)
 k_schur_update(Planes P, StencilArgs a, DevState* st, double* partials) {
     const Blk blk = single_blk();
-    if (st->done) return;
+    if (st->done) {
+        if (first_thread()) report_progress(a, st->iter, 1);
+        return;
+    }
     const int H = a.H, W = a.W, ld = a.ld;
     const int j0 = (blk.bx * kThreads + threadIdx.x) * kVec;
     const int lane = threadIdx.x & 31;
@@ -1477,8 +1495,10 @@ k_schur_update(Planes P, StencilArgs a, DevState* st, double* partials) {
         st->iter = itn;
         const double rel = st->bb > 0.0 ? sqrt(rr_range / st->bb) : 0.0;
         st->rel = rel;
-        if (rel * rel <= a.tol2 || itn >= a.cg_max || !isfinite(rel)) st->done = 1;
+        const bool stop = rel * rel <= a.tol2 || itn >= a.cg_max || !isfinite(rel);
+        if (stop) st->done = 1;
         if (!isfinite(rel)) st->status |= ST_NONFINITE;
+        report_progress(a, itn, stop);
     }
 }
 
