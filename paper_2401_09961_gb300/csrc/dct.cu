@@ -91,6 +91,7 @@ struct QuadArgs {
     DevState* st;
     double* partials;
     int skip_if_done;
+    int pdl;                // dependent launch (host)
 };
 
 // Tiles.  A thread owns MR x NR outputs (row and column groups of four, spread over the tile);
@@ -130,6 +131,7 @@ __device__ __forceinline__ void copy16(float* smem, const float* gmem, bool fill
 
 template <class C, bool SPECTRUM>
 __global__ void __launch_bounds__(C::T, C::MINB) k_quad_gemm_f32(QuadArgs f) {
+    pdl_enter();
     if (f.skip_if_done && f.st->done) return;
     constexpr int BM = C::BM, BN = C::BN, BK = C::BK, RG = C::RG, CG = C::CG;
     extern __shared__ __align__(16) float sm[];
@@ -288,6 +290,7 @@ __global__ void __launch_bounds__(C::T, C::MINB) k_quad_gemm_f32(QuadArgs f) {
 __global__ void __launch_bounds__(256)
 k_quad_fold(const float* __restrict__ R, int ldr, int H, int W, float* __restrict__ Q, int ldq,
             int vec, const DevState* st, int skip_if_done) {
+    pdl_enter();
     if (skip_if_done && st->done) return;
     const int hH = (H + 1) / 2, hW = (W + 1) / 2;
     const int j0 = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
@@ -338,6 +341,7 @@ k_quad_fold(const float* __restrict__ R, int ldr, int H, int W, float* __restric
 __global__ void __launch_bounds__(256)
 k_quad_unfold(const float* __restrict__ Q, int ldq, int H, int W, float* __restrict__ Z, int ldz,
               int vec, const DevState* st, int skip_if_done) {
+    pdl_enter();
     if (skip_if_done && st->done) return;
     const int hH = (H + 1) / 2, hW = (W + 1) / 2;
     const int j0 = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
@@ -456,8 +460,8 @@ static_assert(TileL::SMEM < 47 * 1024 && TileS::SMEM < 47 * 1024 && TileM::SMEM 
 
 template <class C, bool SPECTRUM>
 cudaError_t quad_launch(const QuadArgs& f, cudaStream_t s) {
-    k_quad_gemm_f32<C, SPECTRUM><<<quad_grid<C>(f.M, f.N), C::T, C::SMEM, s>>>(f);
-    return cudaGetLastError();
+    return launch_kernel(f.pdl != 0, k_quad_gemm_f32<C, SPECTRUM>, quad_grid<C>(f.M, f.N), C::T, C::SMEM,
+                         s, f);
 }
 
 // Tile of a launch (0 large, 1 medium, 2 small): the least busy-SM time, in large tiles.  A
@@ -503,13 +507,14 @@ cudaError_t fold_products(const float* R, int ldr, float* Z, int ldz, int H, int
     auto aligned = [&](const float* p, int ld) {
         return W % 4 == 0 && ld % 4 == 0 && (reinterpret_cast<uintptr_t>(p) & 15) == 0;
     };
-    k_quad_fold<<<fold_grid(hH, hW), dim3(64, 4), 0, s>>>(R, ldr, H, W, T1, pw, aligned(R, ldr),
-                                                          base.st, base.skip_if_done);
+    const bool pdl = base.pdl != 0;
+    cudaError_t e = launch_kernel(pdl, k_quad_fold, fold_grid(hH, hW), dim3(64, 4), 0, s, R, ldr, H, W,
+                                  T1, pw, (int)aligned(R, ldr), base.st, base.skip_if_done);
+    if (e != cudaSuccess) return e;
     QuadArgs f = base;
     f.A = T1; f.sa = rows; f.lda = pw; f.B0 = hn.Q0; f.B1 = hn.Q1; f.ldb = ph; f.by_q = 0;
     f.C = T2; f.sc = cols; f.ldc = ph; f.M = hW; f.N = hH; f.K = hH;
-    cudaError_t e = quad_stage<false>(f, s);
-    if (e != cudaSuccess) return e;
+    if ((e = quad_stage<false>(f, s)) != cudaSuccess) return e;
     f.A = T2; f.sa = cols; f.lda = ph; f.B0 = hm.Q0; f.B1 = hm.Q1; f.ldb = pw; f.by_q = 1;
     f.C = T1; f.sc = rows; f.ldc = pw; f.M = hH; f.N = hW; f.K = hW;
     f.n_k = H; f.n_l = W; f.lam_k = lamN; f.lam_l = lamM; f.scale = tau;
@@ -520,9 +525,8 @@ cudaError_t fold_products(const float* R, int ldr, float* Z, int ldz, int H, int
     f.A = T2; f.sa = cols; f.lda = ph; f.B0 = hm.F0; f.B1 = hm.F1; f.ldb = pw; f.by_q = 1;
     f.C = T1; f.sc = rows; f.ldc = pw; f.M = hH; f.N = hW; f.K = hW;
     if ((e = quad_stage<false>(f, s)) != cudaSuccess) return e;
-    k_quad_unfold<<<fold_grid(hH, hW), dim3(64, 4), 0, s>>>(T1, pw, H, W, Z, ldz, aligned(Z, ldz),
-                                                            base.st, base.skip_if_done);
-    return cudaGetLastError();
+    return launch_kernel(pdl, k_quad_unfold, fold_grid(hH, hW), dim3(64, 4), 0, s, T1, pw, H, W, Z, ldz,
+                         (int)aligned(Z, ldz), base.st, base.skip_if_done);
 }
 
 }  // namespace
@@ -593,6 +597,7 @@ cudaError_t dct_apply(const DctPlan& d, const float* rU, float* zU, int ld, DevS
     base.rho = reduce_rho;
     base.flexible = a.flexible;
     base.skip_if_done = skip_if_done;
+    base.pdl = a.pdl;
     return fold_products(rU, ld, zU, ld, d.H, d.W, d.tau, halves(d.halvesN, d.H),
                          halves(d.halvesM, d.W), d.lamN, d.lamM, d.T1, d.T2, base, s);
 }
@@ -624,8 +629,10 @@ cudaError_t dct_apply_fp32_scratch(const float* R, float* Z, int H, int W, float
     if (H != W) k_build_lambda<<<2, 256, 0, s>>>(lamM, W, W);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
+    QuadArgs base{};
+    base.pdl = 1;
     return fold_products(R, W, Z, W, H, W, tau, halves(bn, H), halves(bm, W), lamN, lamM, T1, T2,
-                         QuadArgs{}, s);
+                         base, s);
 }
 
 }  // namespace irls

@@ -755,6 +755,7 @@ k_fftq_rows_fwd(const float* __restrict__ R, float* __restrict__ Tout, int H, in
                 int skip_if_done) {
     using C = RowQ<N>;
     constexpr int GQ = C::GQ;
+    pdl_enter();
     if (skip_if_done && st->done) return;
     extern __shared__ __align__(16) float4 sq[];
     const int row0 = blockIdx.x * 4 * GQ;                // H is a multiple of 4
@@ -813,6 +814,7 @@ k_fftq_cols(float* __restrict__ Tio, int W, int ld, float tau, const float* __re
             int skip_if_done, int flexible) {
     using C = ColQ<N>;
     constexpr int GQ = C::GQ, T = C::T;
+    pdl_enter();
     if (skip_if_done && st->done) return;
     extern __shared__ __align__(16) float4 sq[];
     const int q = threadIdx.x % GQ;                      // T is a multiple of GQ
@@ -906,6 +908,7 @@ k_fftq_rows_inv(const float* __restrict__ Tin, float* __restrict__ Z, int H, int
                 int skip_if_done) {
     using C = RowQ<N>;
     constexpr int GQ = C::GQ;
+    pdl_enter();
     if (skip_if_done && st->done) return;
     extern __shared__ __align__(16) float4 sq[];
     const int row0 = blockIdx.x * 4 * GQ;
@@ -1037,32 +1040,32 @@ cudaError_t prepare_rows() {
 
 template <int N>
 cudaError_t rows_fwd(const float* R, float* Tout, int H, int ld, float tau, const float2* tw,
-                     const float2* tt, const DevState* st, int skip, cudaStream_t s) {
+                     const float2* tt, const DevState* st, int skip, bool pdl, cudaStream_t s) {
     if constexpr (N <= kQuadMaxN) {
         using C = RowQ<N>;
-        k_fftq_rows_fwd<N><<<(H + 4 * C::GQ - 1) / (4 * C::GQ), C::T, C::SMEM, s>>>(
-            R, Tout, H, ld, tau, tw, tt, st, skip);
+        return launch_kernel(pdl, k_fftq_rows_fwd<N>, (H + 4 * C::GQ - 1) / (4 * C::GQ), C::T,
+                             C::SMEM, s, R, Tout, H, ld, tau, tw, tt, st, skip);
     } else {
         using C = RowCfg<N>;
         k_fftdct_rows_fwd<N><<<(H + 2 * C::NF - 1) / (2 * C::NF), C::T, C::SMEM, s>>>(
             R, Tout, H, ld, tau, tw, tt, st, skip);
+        return cudaGetLastError();
     }
-    return cudaGetLastError();
 }
 
 template <int N>
 cudaError_t rows_inv(const float* Tin, float* Z, int H, int ld, const float2* tw, const float2* tt,
-                     const DevState* st, int skip, cudaStream_t s) {
+                     const DevState* st, int skip, bool pdl, cudaStream_t s) {
     if constexpr (N <= kQuadMaxN) {
         using C = RowQ<N>;
-        k_fftq_rows_inv<N><<<(H + 4 * C::GQ - 1) / (4 * C::GQ), C::T, C::SMEM, s>>>(
-            Tin, Z, H, ld, tw, tt, st, skip);
+        return launch_kernel(pdl, k_fftq_rows_inv<N>, (H + 4 * C::GQ - 1) / (4 * C::GQ), C::T,
+                             C::SMEM, s, Tin, Z, H, ld, tw, tt, st, skip);
     } else {
         using C = RowCfg<N>;
         k_fftdct_rows_inv<N><<<(H + 2 * C::NF - 1) / (2 * C::NF), C::T, C::SMEM, s>>>(
             Tin, Z, H, ld, tw, tt, st, skip);
+        return cudaGetLastError();
     }
-    return cudaGetLastError();
 }
 
 template <int N>
@@ -1112,20 +1115,20 @@ cudaError_t fft_dct_apply(const DctPlan& d, const float* rU, float* zU, int ld, 
     if (!d.fft_ready) return cudaErrorInvalidValue;
     const int H = d.H, W = d.W;
     float* T = d.T1;
+    const bool pdl = a.pdl != 0;
     cudaError_t e = with_row_len(W, [&](auto n) {
-        return rows_fwd<n.value>(rU, T, H, ld, d.tau, d.fftTwM, d.fftTtM, st, skip_if_done, s);
+        return rows_fwd<n.value>(rU, T, H, ld, d.tau, d.fftTwM, d.fftTtM, st, skip_if_done, pdl, s);
     });
     if (e != cudaSuccess) return e;
     e = with_col_len(H, [&](auto n) {
         using C = ColQ<n.value>;
-        k_fftq_cols<n.value><<<col_blocks<n.value>(W), C::T, C::SMEM, s>>>(
-            T, W, ld, d.tau, d.lamN, d.lamM, d.fftTwN, d.fftTtN, st, partials, reduce_rho,
-            skip_if_done, a.flexible);
-        return cudaGetLastError();
+        return launch_kernel(pdl, k_fftq_cols<n.value>, col_blocks<n.value>(W), C::T, C::SMEM, s, T,
+                             W, ld, d.tau, d.lamN, d.lamM, d.fftTwN, d.fftTtN, st, partials,
+                             reduce_rho, skip_if_done, a.flexible);
     });
     if (e != cudaSuccess) return e;
     return with_row_len(W, [&](auto n) {
-        return rows_inv<n.value>(T, zU, H, ld, d.fftTwM, d.fftTtM, st, skip_if_done, s);
+        return rows_inv<n.value>(T, zU, H, ld, d.fftTwM, d.fftTtM, st, skip_if_done, pdl, s);
     });
 }
 

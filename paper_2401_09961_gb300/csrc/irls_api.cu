@@ -236,6 +236,7 @@ StencilArgs make_args(const irls_plan_s* p) {
     a.supd_rows = p->supd_rows;
     a.dir_wave = p->dir_wave;
     a.upd_wave = p->upd_wave;
+    a.pdl = p->opts.precision == IRLS_PREC_FP32;
     return a;
 }
 

@@ -499,6 +499,7 @@ __device__ __forceinline__ void k_direction_pap_body(Planes P, StencilArgs a, De
 template <int ROWS>
 __global__ void __launch_bounds__(kThreads)
 k_direction_pap(Planes P, StencilArgs a, DevState* st, double* partials) {
+    pdl_enter();
     k_direction_pap_body<ROWS, false>(P, a, st, partials, single_blk());
 }
 
@@ -669,6 +670,7 @@ __device__ __forceinline__ void k_update_body(Planes P, StencilArgs a, DevState*
 template <int ROWS>
 __global__ void __launch_bounds__(kThreads)
 k_update(Planes P, StencilArgs a, DevState* st, double* partials) {
+    pdl_enter();
     k_update_body<ROWS, false>(P, a, st, partials, single_blk());
 }
 
@@ -1267,6 +1269,7 @@ k_schur_reweight(Planes P, StencilArgs a, DevState* st, double* partials) {
 template <int ROWS>
 __global__ void __launch_bounds__(kThreads)
 k_schur_direction(Planes P, StencilArgs a, DevState* st, double* partials) {
+    pdl_enter();
     const Blk blk = single_blk();
     if (st->done) return;
     const int H = a.H, W = a.W, ld = a.ld;
@@ -1371,6 +1374,7 @@ k_schur_direction(Planes P, StencilArgs a, DevState* st, double* partials) {
 template <int ROWS>
 __global__ void __launch_bounds__(kThreads)
 k_schur_update(Planes P, StencilArgs a, DevState* st, double* partials) {
+    pdl_enter();
     const Blk blk = single_blk();
     if (st->done) {
         if (first_thread()) report_progress(a, st->iter, 1);
@@ -1722,14 +1726,14 @@ cudaError_t launch_rows(int rows, int H, int W, cudaStream_t s, Args... args) {
 template <int R>
 struct DirK {
     static void go(dim3 g, cudaStream_t s, Planes P, StencilArgs a, DevState* st, double* pa) {
-        k_direction_pap<R><<<g, kThreads, 0, s>>>(P, a, st, pa);
+        launch_kernel(a.pdl != 0, k_direction_pap<R>, g, kThreads, 0, s, P, a, st, pa);
     }
 };
 
 template <int R>
 struct UpdK {
     static void go(dim3 g, cudaStream_t s, Planes P, StencilArgs a, DevState* st, double* pa) {
-        k_update<R><<<g, kThreads, 0, s>>>(P, a, st, pa);
+        launch_kernel(a.pdl != 0, k_update<R>, g, kThreads, 0, s, P, a, st, pa);
     }
 };
 
@@ -1802,23 +1806,17 @@ cudaError_t launch_schur_reweight(const Planes& P, const StencilArgs& a, DevStat
 cudaError_t launch_schur_direction(const Planes& P, const StencilArgs& a, DevState* st,
                                    double* partials, cudaStream_t s) {
     const int rows = a.sdir_rows > 0 ? a.sdir_rows : kSchurRows;
-    if (rows == kSchurRows)
-        k_schur_direction<kSchurRows><<<vec_grid(a.H, a.W, rows), kThreads, 0, s>>>(P, a, st,
-                                                                                   partials);
-    else
-        k_schur_direction<0><<<vec_grid(a.H, a.W, rows), kThreads, 0, s>>>(P, a, st, partials);
-    return cudaGetLastError();
+    return launch_kernel(a.pdl != 0,
+                         rows == kSchurRows ? k_schur_direction<kSchurRows> : k_schur_direction<0>,
+                         vec_grid(a.H, a.W, rows), kThreads, 0, s, P, a, st, partials);
 }
 
 cudaError_t launch_schur_update(const Planes& P, const StencilArgs& a, DevState* st,
                                 double* partials, cudaStream_t s) {
     const int rows = a.supd_rows > 0 ? a.supd_rows : kSchurRows;
-    if (rows == kSchurRows)
-        k_schur_update<kSchurRows><<<vec_grid(a.H, a.W, rows), kThreads, 0, s>>>(P, a, st,
-                                                                                partials);
-    else
-        k_schur_update<0><<<vec_grid(a.H, a.W, rows), kThreads, 0, s>>>(P, a, st, partials);
-    return cudaGetLastError();
+    return launch_kernel(a.pdl != 0,
+                         rows == kSchurRows ? k_schur_update<kSchurRows> : k_schur_update<0>,
+                         vec_grid(a.H, a.W, rows), kThreads, 0, s, P, a, st, partials);
 }
 
 cudaError_t launch_schur_recover_v(const Planes& P, const StencilArgs& a, cudaStream_t s) {
