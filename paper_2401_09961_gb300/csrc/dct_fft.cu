@@ -431,9 +431,10 @@ __device__ __forceinline__ void finish_rho_fft(DevState* st, double rho_u, int f
 // straight from global memory and the last one's outputs go straight there.  Per application
 // (caller's arrays, us; one transform a thread before -> quads): 1024^2 47 -> 23, 2048^2 97 -> 44,
 // 4096^2 187 -> 159, 8192^2 1277 -> 773, 4000 x 8000 684 -> 438 (the first two and last two with the
-// plane copies of the time).  At 4096^2 the rows take 33 and 41 us and the columns 85 (ncu) against
-// 20 each for their bytes: shared-memory and L1 wavefronts fill 60 % of the cycles, and 16 warps
-// an SM (128 registers) leave the barriers of the stages exposed.
+// plane copies of the time); with dependent launches and the 2^a 5^3 columns' twiddles in shared
+// memory 4096^2 153, 8192^2 768, 4000 x 8000 416.  At 4096^2 the rows take 32 and 42 us and the
+// columns 84 (ncu) against 20 each for their bytes: shared-memory and L1 wavefronts fill 60 % of the
+// cycles, and 16 warps an SM (128 registers) leave the barriers of the stages exposed.
 typedef unsigned long long u64;
 struct Cq { u64 re, im; };   // two complex values: (re0, re1), (im0, im1)
 
@@ -597,14 +598,17 @@ __host__ __device__ constexpr int quad_radix(int N, int NS) {
     if (N % 5 == 0) return rem == 100 ? 10 : rem % 20 == 0 ? 20 : rem;
     return rem % 16 == 0 ? 16 : rem;
 }
-// Shape of a quad launch: GQ quads a block, one thread per first-stage butterfly of a quad.
-template <int N, int GQ_>
+// Shape of a quad launch: GQ quads a block, one thread per first-stage butterfly of a quad; with
+// TWS the stages' twiddles lie in shared memory behind the quads.
+template <int N, int GQ_, bool TWS_ = false>
 struct QuadShape {
     static constexpr int GQ = GQ_;
     static constexpr int PADB = N % 5 == 0 ? 20 : 16;
     static constexpr int T = (N / quad_radix(N, 1) * GQ + 31) / 32 * 32;
     static constexpr int ROWS = N + N / PADB;             // 16-byte rows of a quad
-    static constexpr size_t SMEM = (size_t)ROWS * GQ * 16;
+    static constexpr bool TWS = TWS_;
+    static constexpr int TWN = N - quad_radix(N, 1);      // twiddles of all stages
+    static constexpr size_t SMEM = (size_t)ROWS * GQ * 16 + (TWS ? TWN * sizeof(float2) : 0);
     static constexpr int MINB = 512 / T < 1 ? 1 : (512 / T > 8 ? 8 : 512 / T);
     // the last stage: its sub-transform length, radix and butterflies a thread
     static constexpr int last_ns() {
@@ -618,11 +622,15 @@ struct QuadShape {
 };
 // Rows: enough threads a block at short lengths.  Columns: at least two quads (a whole 32-byte
 // sector of each image row) where they fit shared memory: 4096^2 159 us an application, 165 with
-// one quad and two blocks an SM; 2048^2 44 against 48.
+// one quad and two blocks an SM; 2048^2 44 against 48.  The 2^a 5^3 columns take their twiddles from
+// shared memory: one block an SM leaves room for them, while in L1 the image's sectors drive them out
+// (a fifth of its reads hit): columns of 4000 x 8000 212 to 198 us, of 8000 x 4000 260 to 233, of
+// 4000^2 with the rows 212 to 207.  The powers of two lose by it (4096^2 84 to 90, 8192^2 399 to
+// 525), 2000 gains nothing (27.5 to 27.9), and rows lose (8000 x 4000 92 to 98).
 template <int N>
 using RowQ = QuadShape<N, N >= 1000 ? 1 : N >= 512 ? 2 : N >= 256 ? 4 : 8>;
 template <int N>
-using ColQ = QuadShape<N, N >= 5000 ? 1 : N >= 1000 ? 2 : N >= 512 ? 4 : 8>;
+using ColQ = QuadShape<N, N >= 5000 ? 1 : N >= 1000 ? 2 : N >= 512 ? 4 : 8, N % 5 == 0 && N >= 4000>;
 constexpr int kQuadMaxN = 8192;
 // Lengths whose first stage loads its inputs itself; a radix-20 butterfly has no registers left for
 // the addresses, so the 2^a 5^3 lengths bring theirs in through shared memory.
@@ -643,6 +651,19 @@ __device__ __forceinline__ Cq qld(const float4* p) {
 __device__ __forceinline__ void qst(float4* p, Cq v) {
     *reinterpret_cast<ulonglong2*>(p) = make_ulonglong2(v.re, v.im);
 }
+// The stages' twiddles as quad_stages takes them: in shared memory behind the quads (asynchronous
+// copies, complete at the cp.async.wait_all and barrier before the first stage) or where they are.
+template <class C>
+__device__ __forceinline__ const float2* stage_twiddles(float4* sq, const float2* __restrict__ tw) {
+    if constexpr (C::TWS) {
+        static_assert(C::TWN % 2 == 0, "whole 16-byte pieces");
+        float4* t = sq + C::ROWS * C::GQ;
+        for (int e = threadIdx.x; e < C::TWN / 2; e += C::T) cp_async16(t + e, tw + 2 * e, true);
+        return reinterpret_cast<const float2*>(t);
+    } else {
+        return tw;
+    }
+}
 struct FromShared {};   // the first stage's inputs are in the block's rows
 
 // Stockham stages from sub-transform length NS on, in the block's rows s (tw: this stage's table).
@@ -650,7 +671,7 @@ struct FromShared {};   // the first stage's inputs are in the block's rows
 // leaves its outputs in `o`: o[b][r] is element j + r LNS of quad q for b's (q, j).  So neither the
 // loads nor the stores of a transform pass through shared memory.
 template <int N, class C, int NS, class First>
-__device__ __forceinline__ void quad_stages(float4* s, const float2* __restrict__ tw, First first,
+__device__ __forceinline__ void quad_stages(float4* s, const float2* tw, First first,
                                             Cq (&o)[C::LPER][C::LR]) {
     constexpr int R = quad_radix(N, NS), NJ = N / R, NB = NJ * C::GQ, T = C::T;
     constexpr int PER = (NB + T - 1) / T, GQ = C::GQ;
@@ -683,7 +704,8 @@ __device__ __forceinline__ void quad_stages(float4* s, const float2* __restrict_
             if constexpr (NS > 1) {
 #pragma unroll
                 for (int r = 1; r < R; ++r) {
-                    const float2 w = __ldg(&tw[(r - 1) * NS + k]);
+                    const float2* p = &tw[(r - 1) * NS + k];
+                    const float2 w = C::TWS ? *p : __ldg(p);
                     v[b][r] = qmul(v[b][r], w.x, w.y);
                 }
             }
@@ -821,9 +843,11 @@ k_fftq_cols(float* __restrict__ Tio, int W, int ld, float tau, const float* __re
     const int j0 = (blockIdx.x * GQ + q) * 4;
     const bool in = j0 < W;                              // W is a multiple of 4
     const float4 m = in ? __ldg(reinterpret_cast<const float4*>(lamM + j0)) : make_float4(1.f, 1.f, 1.f, 1.f);
+    const float2* tws = stage_twiddles<C>(sq, tw);
+    static_assert(!C::TWS || !quad_direct(N), "the copies are waited for with the columns'");
     Cq o[C::LPER][C::LR];
     if constexpr (quad_direct(N)) {
-        quad_stages<N, C, 1>(sq, tw, [&](int, int j, int r, int NJ) {
+        quad_stages<N, C, 1>(sq, tws, [&](int, int j, int r, int NJ) {
             const int i = source_of<N, quad_radix(N, 1)>(j, r, NJ);
             if (!in) return Cq{0ull, 0ull};
             const ulonglong2 x = *reinterpret_cast<const ulonglong2*>(Tio + ((unsigned)i * ld + j0));
@@ -837,7 +861,7 @@ k_fftq_cols(float* __restrict__ Tio, int W, int ld, float tau, const float* __re
         }
         asm volatile("cp.async.wait_all;\n" ::: "memory");
         __syncthreads();
-        quad_stages<N, C, 1>(sq, tw, FromShared(), o);
+        quad_stages<N, C, 1>(sq, tws, FromShared(), o);
     }
     __syncthreads();
     quad_outputs<C>(o, [&](Cq& z, int, int j, int r) { qst(sq + C::slot(j + r * C::LNS) * GQ + q, z); });
@@ -883,7 +907,7 @@ k_fftq_cols(float* __restrict__ Tio, int W, int ld, float tau, const float* __re
         }
     }
     __syncthreads();
-    quad_stages<N, C, 1>(sq, tw, FromShared(), o);
+    quad_stages<N, C, 1>(sq, tws, FromShared(), o);
     if (in)
         quad_outputs<C>(o, [&](Cq& z, int, int j, int r) {
             const int i = source_of<N, C::LR>(j, r, C::LNS);
