@@ -529,6 +529,190 @@ cudaError_t fold_products(const float* R, int ldr, float* Z, int ldz, int H, int
                          (int)aligned(Z, ldz), base.st, base.skip_if_done);
 }
 
+// ---- full-size products, for taped solves and their adjoint -----------------------------------
+// The gradient divides by W = sqrt(C^2 V^2 + delta^2) of edges whose V is close to zero, so it
+// carries the rounding of the solves times up to 1 / delta: 1e-7 of z_U, where the quadrant
+// products round otherwise than the full ones, moves dL/dX by 1e-4 (both as far from the float64
+// gradient; with the full-size products two versions of the library agree to 2e-7).  So that
+// gradients do not move, the solves that a tape records and the adjoint's keep the full-size
+// products and their order of summation: T1 = R P_M, T2 = (T1^T P_N) scaled, T1 = T2 P_N^T,
+// Z = T1 P_M^T, each output one chain of multiply-adds along k.  128 x 128 tiles, 8 x 8 a thread,
+// operands staged through registers: 43 TFLOP/s at 4096^2, of twice the quadrants' work.  A
+// recorded solve with its adjoint at 486 x 931, four steps: 595 ms (quadrants: about 190).
+constexpr int kFullTile = 128;
+
+enum Epi : int { EPI_TRANS = 0, EPI_EIG = 1, EPI_ZU = 2, EPI_ZU_RHO = 3 };
+
+struct EpiArgs {
+    float* C;          // output
+    int ldc;
+    int vm, vn;        // valid extents (EPI_EIG: W, H; EPI_ZU: H, W)
+    const float* lam_m;
+    const float* lam_n;
+    float scale;       // tau (EPI_EIG)
+    const float* rU;   // EPI_ZU_RHO: residual plane, pitch ldc
+    DevState* st;
+    double* partials;
+    int flexible;
+};
+
+// C[m][n] = sum_k A[m][k] B[n][k], M and N multiples of 128; A rows >= a_rows and k >= K read 0.
+template <int EPI>
+__global__ void __launch_bounds__(256)
+k_gemm_tn_f32(const float* __restrict__ A, int lda, int a_rows, const float* __restrict__ B,
+              int ldb, int K, EpiArgs ep, int skip_if_done) {
+    if (skip_if_done && ep.st != nullptr && ep.st->done) return;
+    constexpr int BM = kFullTile, BN = kFullTile, BK = 8;
+    __shared__ __align__(16) float As[2][BK][BM + 4];
+    __shared__ __align__(16) float Bs[2][BK][BN + 4];
+    const int tid = threadIdx.x;
+    const int tx = tid & 15, ty = tid >> 4;
+    const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
+    // loader mapping: 128 rows x 8 k per operand; thread -> (row, 4 consecutive k)
+    const int lr = tid >> 1, lk = (tid & 1) * 4;
+    const bool arow = (m0 + lr) < a_rows;
+    const float* Ap = A + (size_t)(m0 + lr) * lda;
+    const float* Bp = B + (size_t)(n0 + lr) * ldb;
+
+    auto load4 = [&](const float* p, bool rowok, int k, float (&r)[4]) {
+        if (rowok && k + 3 < K) {
+            float4 v = *reinterpret_cast<const float4*>(p + k);
+            r[0] = v.x; r[1] = v.y; r[2] = v.z; r[3] = v.w;
+        } else {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) r[c] = (rowok && k + c < K) ? p[k + c] : 0.f;
+        }
+    };
+
+    float ra[4], rb[4];
+    load4(Ap, arow, lk, ra);
+    load4(Bp, true, lk, rb);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) { As[0][lk + c][lr] = ra[c]; Bs[0][lk + c][lr] = rb[c]; }
+    __syncthreads();
+
+    float acc[8][8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
+
+    const int nk = (K + BK - 1) / BK;
+    for (int kt = 0; kt < nk; ++kt) {
+        const int buf = kt & 1;
+        if (kt + 1 < nk) {
+            load4(Ap, arow, (kt + 1) * BK + lk, ra);
+            load4(Bp, true, (kt + 1) * BK + lk, rb);
+        }
+#pragma unroll
+        for (int kk = 0; kk < BK; ++kk) {
+            const float4 a0 = *reinterpret_cast<const float4*>(&As[buf][kk][ty * 4]);
+            const float4 a1 = *reinterpret_cast<const float4*>(&As[buf][kk][64 + ty * 4]);
+            const float4 b0 = *reinterpret_cast<const float4*>(&Bs[buf][kk][tx * 4]);
+            const float4 b1 = *reinterpret_cast<const float4*>(&Bs[buf][kk][64 + tx * 4]);
+            const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+            const float bv[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+#pragma unroll
+                for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
+        }
+        if (kt + 1 < nk) {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                As[buf ^ 1][lk + c][lr] = ra[c];
+                Bs[buf ^ 1][lk + c][lr] = rb[c];
+            }
+        }
+        __syncthreads();
+    }
+
+    CSum part;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int m = m0 + (i < 4 ? ty * 4 + i : 64 + ty * 4 + (i - 4));
+        float row = 0.f;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const int n = n0 + (j < 4 ? tx * 4 + j : 64 + tx * 4 + (j - 4));
+            const float v = acc[i][j];
+            if constexpr (EPI == EPI_TRANS) {
+                ep.C[(size_t)n * ep.ldc + m] = v;
+            } else if constexpr (EPI == EPI_EIG) {
+                float o = 0.f;
+                if (m < ep.vm && n < ep.vn && (m | n) != 0) o = ep.scale * v / (ep.lam_m[m] + ep.lam_n[n]);
+                ep.C[(size_t)m * ep.ldc + n] = o;
+            } else {
+                if (m < ep.vm && n < ep.vn) {
+                    ep.C[(size_t)m * ep.ldc + n] = v;
+                    if constexpr (EPI == EPI_ZU_RHO) row += ep.rU[(size_t)m * ep.ldc + n] * v;
+                }
+            }
+        }
+        if constexpr (EPI == EPI_ZU_RHO) part.add(row);
+    }
+    if constexpr (EPI == EPI_ZU_RHO) {
+        double vv[1] = {part.value()}, tot[1];
+        const Blk blk = single_blk();
+        if (grid_reduce<1>(vv, ep.partials, &ep.st->counter, tot, blk.nblk, blk.bid) && tid == 0)
+            finish_rho(ep.st, tot[0], ep.flexible);
+    }
+}
+
+// P[i][k] = c_k cos(pi k (2i+1) / (2N)) and its transpose, zero-padded to Np x Np.  The
+// argument is reduced exactly in integers before the FP64 cospi.
+__global__ void k_build_full(float* P, float* PT, int N, int Np) {
+    const size_t total = (size_t)Np * Np;
+    for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < total;
+         t += (size_t)gridDim.x * blockDim.x) {
+        const int i = (int)(t / Np), k = (int)(t % Np);
+        double v = 0.0;
+        if (i < N && k < N) {
+            const long long m = ((long long)(2 * i + 1) * k) % (4LL * N);
+            const double ck = k == 0 ? sqrt(1.0 / N) : sqrt(2.0 / N);
+            v = ck * cospi((double)m / (2.0 * N));
+        }
+        P[(size_t)i * Np + k] = (float)v;
+        PT[(size_t)k * Np + i] = (float)v;
+    }
+}
+
+template <int EPI>
+cudaError_t full_gemm(const float* A, int lda, int a_rows, const float* B, int ldb, int M, int N,
+                      int K, const EpiArgs& ep, int skip, cudaStream_t s) {
+    dim3 grid(N / kFullTile, M / kFullTile);
+    k_gemm_tn_f32<EPI><<<grid, 256, 0, s>>>(A, lda, a_rows, B, ldb, K, ep, skip);
+    return cudaGetLastError();
+}
+
+cudaError_t full_products(const DctPlan& d, const float* rU, float* zU, int ld, DevState* st,
+                          int reduce_rho, int flexible, double* partials, int skip,
+                          cudaStream_t s) {
+    const int H = d.H, W = d.W, Hp = d.Hp, Wp = d.Wp;
+    cudaError_t e;
+    EpiArgs ep{};
+    ep.st = st;
+    ep.partials = partials;
+    ep.flexible = flexible;
+    // stage 1: T1[l][i] = sum_j R[i][j] PMT[l][j]
+    ep.C = d.T1; ep.ldc = Hp;
+    e = full_gemm<EPI_TRANS>(rU, ld, H, d.PMT, Wp, Hp, Wp, W, ep, skip, s);
+    if (e != cudaSuccess) return e;
+    // stage 2: T2[l][k] = tau sum_i T1[l][i] PNT[k][i] / (m_l + l_k), (0,0) -> 0
+    ep.C = d.T2; ep.ldc = Hp; ep.vm = W; ep.vn = H; ep.lam_m = d.lamM; ep.lam_n = d.lamN;
+    ep.scale = d.tau;
+    e = full_gemm<EPI_EIG>(d.T1, Hp, Wp, d.PNT, Hp, Wp, Hp, H, ep, skip, s);
+    if (e != cudaSuccess) return e;
+    // stage 3: T1[i][l] = sum_k T2[l][k] PN[i][k]
+    ep.C = d.T1; ep.ldc = Wp;
+    e = full_gemm<EPI_TRANS>(d.T2, Hp, Wp, d.PN, Hp, Wp, Hp, H, ep, skip, s);
+    if (e != cudaSuccess) return e;
+    // stage 4: Z[i][j] = sum_l T1[i][l] PM[j][l]
+    ep.C = zU; ep.ldc = ld; ep.vm = H; ep.vn = W; ep.rU = rU;
+    return reduce_rho ? full_gemm<EPI_ZU_RHO>(d.T1, Wp, Hp, d.PM, Wp, Hp, Wp, W, ep, skip, s)
+                      : full_gemm<EPI_ZU>(d.T1, Wp, Hp, d.PM, Wp, Hp, Wp, W, ep, skip, s);
+}
+
 }  // namespace
 
 // blocks of the grid-reduced second product in its smallest tile
@@ -580,7 +764,31 @@ cudaError_t dct_setup(DctPlan& d, int H, int W, int prec, float tau, char* mem) 
     return e;
 }
 
-void dct_release(DctPlan& d) { umma_dct_release(d); }
+void dct_release(DctPlan& d) {
+    if (d.full_mem) cudaFree(d.full_mem);
+    d.full_mem = nullptr;
+    umma_dct_release(d);
+}
+
+// The full-size bases of the float32 dense form, on the first solve of a plan that needs them
+// (kept with the plan).  Nothing for the other forms.
+cudaError_t dct_full_setup(DctPlan& d, cudaStream_t s) {
+    if (d.full_mem || d.fft || d.prec != IRLS_PREC_FP32) return cudaSuccess;
+    const size_t n = (size_t)d.Hp * d.Hp, m = d.H != d.W ? (size_t)d.Wp * d.Wp : 0;
+    cudaError_t e = cudaMalloc(&d.full_mem, 2 * (n + m) * sizeof(float));
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        d.full_mem = nullptr;
+        return e;
+    }
+    d.PN = static_cast<float*>(d.full_mem);
+    d.PNT = d.PN + n;
+    d.PM = m ? d.PNT + n : d.PN;
+    d.PMT = m ? d.PM + m : d.PNT;
+    k_build_full<<<1024, 256, 0, s>>>(d.PN, d.PNT, d.H, d.Hp);
+    if (m) k_build_full<<<1024, 256, 0, s>>>(d.PM, d.PMT, d.W, d.Wp);
+    return cudaGetLastError();
+}
 cudaError_t dct_reset(const DctPlan& d, cudaStream_t s) { return umma_dct_reset(d, s); }
 bool dct_stall(DctPlan& d, int on) { return umma_dct_stall(d, on); }
 
@@ -591,6 +799,8 @@ cudaError_t dct_apply(const DctPlan& d, const float* rU, float* zU, int ld, DevS
     if (d.prec != IRLS_PREC_FP32)
         return umma_dct_apply(d, rU, zU, ld, st, reduce_rho, a, partials, skip_if_done, s, src,
                               ld_src);
+    if (a.full)
+        return full_products(d, rU, zU, ld, st, reduce_rho, a.flexible, partials, skip_if_done, s);
     QuadArgs base{};
     base.st = st;
     base.partials = partials;

@@ -109,7 +109,7 @@ enum ProfClass : int {
 };
 
 // Records an event pair around each profiled launch and folds the elapsed times in once the
-// stream has passed them (the solve already waits on chunk boundaries, so draining adds no
+// stream has passed them (the solve waits for the device's progress anyway, so draining adds no
 // synchronisation of its own).
 struct Profiler {
     bool on = false;
@@ -379,7 +379,8 @@ int run_solve(irls_plan_s* p, const float* X, const float* coh, const float* Cv,
               const float* U0, const float* Vv0, const float* Vh0, cudaStream_t s,
               irls_stats* stats, irls_tape_s* tape = nullptr) {
     TraceRange trace("irls_unwrap");
-    const StencilArgs a = make_args(p);
+    StencilArgs a = make_args(p);
+    a.full = tape != nullptr;
     DevState* st = p->st;
     Profiler& pf = p->prof;
     const size_t pb = p->L.plane_bytes;
@@ -986,6 +987,13 @@ int irls_unwrap_forward_record(irls_plan p, const float* X, const float* coh, co
         float* f[64 + 2 * IRLS_MAX_OUTER];
         for (size_t i = 0; i < nplanes; ++i)
             f[i] = reinterpret_cast<float*>(t->mem + i * t->plane_bytes);
+        if (cudaError_t e = dct_full_setup(p->dct, s); e == cudaErrorMemoryAllocation) {
+            cudaFree(t->mem);
+            delete t;
+            return IRLS_ERR_OOM;
+        } else {
+            ck(e);
+        }
         size_t q = 0;
         t->Gv = f[q++]; t->Gh = f[q++]; t->Cv = f[q++]; t->Ch = f[q++];
         t->Gbv = f[q++]; t->Gbh = f[q++]; t->Cbv = f[q++]; t->Cbh = f[q++];
@@ -1020,7 +1028,12 @@ int irls_unwrap_backward(irls_tape t, const float* dLdU, float* dLdX, float* dLd
     int status = 0;
     try {
         DeviceGuard g(p->dev);
-        const StencilArgs a = make_args(p);
+        StencilArgs a = make_args(p);
+        a.full = 1;
+        if (cudaError_t e = dct_full_setup(p->dct, s); e == cudaErrorMemoryAllocation)
+            return IRLS_ERR_OOM;
+        else
+            ck(e);
         DevState* st = p->st;
         const size_t pb = t->plane_bytes;
         ck(cudaMemsetAsync(st, 0, sizeof(DevState), s));

@@ -124,6 +124,7 @@ struct StencilArgs {
     unsigned long long* progress;
     unsigned epoch;
     int pdl;   // dependent launches within a CG iteration (host; see pdl_enter)
+    int full;  // float32 dense products at full size (host; a taped solve or its adjoint)
 };
 
 // Rows of a summation unit for a tile of `rows` rows and a one-wave count of `wave` rows, and the
@@ -157,6 +158,9 @@ struct DctPlan {
     float *halvesN, *halvesM;
     float *lamN, *lamM;     // eigenvalues, padded with zeros
     float *T1, *T2;         // fp32 intermediates (Wp x Hp each)
+    // full-size fp32 bases and transposes (Hp^2, Wp^2; taped solves only, see dct_full_setup)
+    float *PN, *PNT, *PM, *PMT;
+    void* full_mem;
     // bfloat16 copies for the tensor-core path (the *lo parts only in split precision)
     void *PN16, *PNT16, *PM16, *PMT16;
     void *PN16lo, *PNT16lo, *PM16lo, *PMT16lo;
@@ -324,6 +328,7 @@ cudaError_t dct_setup(DctPlan& d, int H, int W, int prec, float tau, char* mem);
 // receives error flags; with reduce_rho the last GEMM also forms rho = r_U^T z_U + st->rz_v
 // and the next beta (Alg. 2).  With skip_if_done the launches return at once once CG stopped.
 void dct_release(DctPlan& d);
+cudaError_t dct_full_setup(DctPlan& d, cudaStream_t s);
 // zeroes the folded form's launch counters (recovery after a launch that timed out)
 cudaError_t dct_reset(const DctPlan& d, cudaStream_t s);
 // test hook: the folded launch's dependency waits run out (IRLS_ERR_TIMEOUT path)
