@@ -445,8 +445,9 @@ def main():
                                "frac_of_hbm": bytes_px[c] * P / t / 1e9 / peaks["hbm_gbs"]})
     per_cls["_pass"] = f"{prof_steps} unwraps with the live per-class profiler on, after the timed region"
     # multiply-adds the preconditioner performs per application: four n^3 products in the direct
-    # form; the folded form runs each stage as half-size products (half of that)
-    dct_flops = 4.0 * n * wd * (n + wd) * (0.5 if folded else 1.0)
+    # form; the folded form and the float32 dense form run each stage as half-size products
+    # (half of that)
+    dct_flops = 4.0 * n * wd * (n + wd) * (0.5 if folded or prec == "fp32" else 1.0)
     dom = max(("direction_pap", "update", "dct_precond", "reweight_residual"),
               key=lambda c: per_cls[c]["ms"])
     avg_s = per_cls[dom]["ms"] / 1e3 / max(live[dom], 1)
@@ -454,7 +455,7 @@ def main():
         if prec == "fp32":
             clk_mhz = clk.get("sm_mhz") or 1900.0
             peak = 152 * 128 * 2 * clk_mhz * 1e6 / 1e12
-            roof = {"kernel": "dct_precond (4 SIMT fp32 GEMMs)", "bound": "alu",
+            roof = {"kernel": "dct_precond (fp32 quadrant products, FMA pipe)", "bound": "alu",
                     "achieved": dct_flops / avg_s / 1e12, "peak": peak, "unit": "TFLOP/s",
                     "peak_source": f"152 SMs x 128 fp32 lanes x 2 x {clk_mhz:.0f} MHz (derived)"}
         else:

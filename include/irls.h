@@ -166,7 +166,7 @@ int irls_plan_set_opts(irls_plan plan, const irls_opts* opts);
 
 /* Preconditioner form the plan runs with its current options: IRLS_DCT_FOLDED or
  * IRLS_DCT_DIRECT for the tensor-core precisions, IRLS_DCT_FFT for the fast-transform form,
- * IRLS_DCT_AUTO for IRLS_PREC_FP32 with dense products (float32 SIMT GEMMs, no tensor cores);
+ * IRLS_DCT_AUTO for IRLS_PREC_FP32 with dense products (float32 FMA, no tensor cores);
  * IRLS_ERR_ARG for a NULL plan.  The paper has no counterpart (an implementation
  * choice of this library). */
 int irls_plan_dct_form(irls_plan plan);
@@ -174,8 +174,9 @@ int irls_plan_dct_form(irls_plan plan);
 /* Tile shapes of the CG direction and update kernels (Alg. 2's two stencil passes per
  * iteration, both bound by HBM bandwidth): image rows per thread block, 8 to 64 for a plan
  * (defaults 24 and 32; batches: one of 8, 16, 24, 32, see irls_batch_set_tiles), or fewer where
- * a small image's launch would otherwise leave SMs idle.  They change the block decomposition, so results change within rounding (the reductions' summation order
- * follows the blocks), never the method.  irls_plan_set_tiles sets them (0 keeps a value;
+ * a small image's launch would otherwise leave SMs idle.  They change the block decomposition, so
+ * results change within rounding (the reductions' summation order follows the blocks), never the
+ * method.  irls_plan_set_tiles sets them (0 keeps a value;
  * anything outside 8..64 is IRLS_ERR_ARG); irls_plan_get_tiles reads the values in use.
  * irls_plan_autotune times, for each kernel, 8, 16, 24 and 32 rows and the row counts that make
  * the kernel's launch the fewest whole waves on this device with at most 32 and at most 64 rows

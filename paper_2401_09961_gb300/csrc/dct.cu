@@ -538,7 +538,8 @@ cudaError_t fold_products(const float* R, int ldr, float* Z, int ldz, int H, int
 // products and their order of summation: T1 = R P_M, T2 = (T1^T P_N) scaled, T1 = T2 P_N^T,
 // Z = T1 P_M^T, each output one chain of multiply-adds along k.  128 x 128 tiles, 8 x 8 a thread,
 // operands staged through registers: 43 TFLOP/s at 4096^2, of twice the quadrants' work.  A
-// recorded solve with its adjoint at 486 x 931, four steps: 595 ms (quadrants: about 190).
+// recorded solve with its adjoint at 486 x 931, four steps, takes 595 ms (679 before the stencils'
+// one-wave rows and the dependent launches).
 constexpr int kFullTile = 128;
 
 enum Epi : int { EPI_TRANS = 0, EPI_EIG = 1, EPI_ZU = 2, EPI_ZU_RHO = 3 };
