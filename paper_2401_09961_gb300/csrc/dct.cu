@@ -141,8 +141,8 @@ __global__ void __launch_bounds__(C::T, C::MINB) k_quad_gemm_f32(QuadArgs f) {
     const int tx = (wg % (C::TX / 8)) * 8 + (lane & 7), ty = (wg / (C::TX / 8)) * 4 + (lane >> 3);
     const int z = blockIdx.z, s = z & 1, q = z >> 1;
     const int m_blk = blockIdx.y * BM, n_blk = blockIdx.x * BN;
-    const float* __restrict__ A = f.A + z * f.sa;
-    const float* __restrict__ B = (f.by_q ? q : s) ? f.B1 : f.B0;
+    const float* A = f.A + z * f.sa;
+    const float* B = (f.by_q ? q : s) ? f.B1 : f.B0;
 
     auto load = [&](int kt) {
         float* buf = sm + (kt % C::ST) * C::BUF;
@@ -288,16 +288,16 @@ __global__ void __launch_bounds__(C::T, C::MINB) k_quad_gemm_f32(QuadArgs f) {
 // Quadrant planes of R (pitch ldr) into Q (four planes hH x ldq): a thread takes four columns of
 // a row pair and their mirrors.  Bound by memory: 4 bytes a pixel read and written.
 __global__ void __launch_bounds__(256)
-k_quad_fold(const float* __restrict__ R, int ldr, int H, int W, float* __restrict__ Q, int ldq,
-            int vec, const DevState* st, int skip_if_done) {
+k_quad_fold(const float* R, int ldr, int H, int W, float* __restrict__ Q, int ldq, int vec,
+            const DevState* st, int skip_if_done) {
     pdl_enter();
     if (skip_if_done && st->done) return;
     const int hH = (H + 1) / 2, hW = (W + 1) / 2;
     const int j0 = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
     const int i = blockIdx.y * blockDim.y + threadIdx.y;
     if (i >= hH || j0 >= ldq) return;
-    const float* __restrict__ up = R + (size_t)i * ldr;
-    const float* __restrict__ dn = R + (size_t)(H - 1 - i) * ldr;
+    const float* up = R + (size_t)i * ldr;
+    const float* dn = R + (size_t)(H - 1 - i) * ldr;
     float a[4] = {0, 0, 0, 0}, b[4] = {0, 0, 0, 0}, c[4] = {0, 0, 0, 0}, d[4] = {0, 0, 0, 0};
     if (vec && j0 + 3 < hW) {
         const float4 x = *reinterpret_cast<const float4*>(up + j0);
@@ -339,7 +339,7 @@ k_quad_fold(const float* __restrict__ R, int ldr, int H, int W, float* __restric
 
 // Z (pitch ldz) from its quadrant planes (hH x ldq each).
 __global__ void __launch_bounds__(256)
-k_quad_unfold(const float* __restrict__ Q, int ldq, int H, int W, float* __restrict__ Z, int ldz,
+k_quad_unfold(const float* Q, int ldq, int H, int W, float* __restrict__ Z, int ldz,
               int vec, const DevState* st, int skip_if_done) {
     pdl_enter();
     if (skip_if_done && st->done) return;

@@ -772,7 +772,7 @@ __device__ __forceinline__ void quad_inverse(u64 yk, u64 zk, u64 yp, u64 zp, flo
 // ---- rows, forward (quads): T[i][k] = tau * sum_j r_U[i][j] P_M[j][k] ------------------------
 template <int N>
 __global__ void __launch_bounds__(RowQ<N>::T, RowQ<N>::MINB)
-k_fftq_rows_fwd(const float* __restrict__ R, float* __restrict__ Tout, int H, int ld, float tau,
+k_fftq_rows_fwd(const float* R, float* __restrict__ Tout, int H, int ld, float tau,
                 const float2* __restrict__ tw, const float2* __restrict__ tt, const DevState* st,
                 int skip_if_done) {
     using C = RowQ<N>;
@@ -787,8 +787,7 @@ k_fftq_rows_fwd(const float* __restrict__ R, float* __restrict__ Tout, int H, in
             // (planes hold less than 2^31 elements: 32-bit offsets from a uniform base)
             const unsigned e = (unsigned)min(row0 + 4 * q, H - 4) * ld +
                                source_of<N, quad_radix(N, 1)>(j, r, NJ);
-            return Cq{pk(__ldg(R + e), __ldg(R + e + ld)),
-                      pk(__ldg(R + e + 2u * ld), __ldg(R + e + 3u * ld))};
+            return Cq{pk(R[e], R[e + ld]), pk(R[e + 2u * ld], R[e + 3u * ld])};
         }, o);
     } else {
         // four columns of four rows a thread, transposed into the rows of the even/odd reordering
@@ -797,7 +796,7 @@ k_fftq_rows_fwd(const float* __restrict__ R, float* __restrict__ Tout, int H, in
             const unsigned e = (unsigned)min(row0 + 4 * q, H - 4) * ld + n;
             float4 x[4];
 #pragma unroll
-            for (int c = 0; c < 4; ++c) x[c] = __ldg(reinterpret_cast<const float4*>(R + e + c * ld));
+            for (int c = 0; c < 4; ++c) x[c] = *reinterpret_cast<const float4*>(R + e + c * ld);
             float4* p = sq + q;
             p[C::slot(reorder_pos<N>(n)) * GQ] = make_float4(x[0].x, x[1].x, x[2].x, x[3].x);
             p[C::slot(reorder_pos<N>(n + 1)) * GQ] = make_float4(x[0].y, x[1].y, x[2].y, x[3].y);
@@ -927,7 +926,7 @@ k_fftq_cols(float* __restrict__ Tio, int W, int ld, float tau, const float* __re
 // four rows, from the row itself at k and N-k.
 template <int N>
 __global__ void __launch_bounds__(RowQ<N>::T, RowQ<N>::MINB)
-k_fftq_rows_inv(const float* __restrict__ Tin, float* __restrict__ Z, int H, int ld,
+k_fftq_rows_inv(const float* Tin, float* __restrict__ Z, int H, int ld,
                 const float2* __restrict__ tw, const float2* __restrict__ tt, const DevState* st,
                 int skip_if_done) {
     using C = RowQ<N>;
@@ -947,10 +946,10 @@ k_fftq_rows_inv(const float* __restrict__ Tin, float* __restrict__ Z, int H, int
         // (Y_0 - i 0) sqrt(1/N) without the half: the factor of k = 0
         const float tx = zero ? dct_c<N>(0) : 0.5f * c * t.x, ty = zero ? 0.f : 0.5f * c * t.y;
         const u64 px = pk(tx), nx = pk(zero ? 0.f : -tx), ny = pk(-ty);
-        const u64 yk = pk(__ldg(Tin + p), __ldg(Tin + p + ld));
-        const u64 zk = pk(__ldg(Tin + p + 2u * ld), __ldg(Tin + p + 3u * ld));
-        const u64 yp = pk(__ldg(Tin + n), __ldg(Tin + n + ld));
-        const u64 zp = pk(__ldg(Tin + n + 2u * ld), __ldg(Tin + n + 3u * ld));
+        const u64 yk = pk(Tin[p], Tin[p + ld]);
+        const u64 zk = pk(Tin[p + 2u * ld], Tin[p + 3u * ld]);
+        const u64 yp = pk(Tin[n], Tin[n + ld]);
+        const u64 zp = pk(Tin[n + 2u * ld], Tin[n + 3u * ld]);
         const u64 ar = pfma(yp, ny, pmul(yk, px)), ai = pfma(yk, ny, pmul(yp, nx));
         const u64 br = pfma(zp, ny, pmul(zk, px)), bi = pfma(zk, ny, pmul(zp, nx));
         return Cq{psub(ar, bi), pneg(padd(ai, br))};

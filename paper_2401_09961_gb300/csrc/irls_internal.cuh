@@ -225,7 +225,10 @@ struct BatchDctPlan {
 // Programmatic dependent launch within a CG iteration of the float32 forms (direction,
 // preconditioner, update): the next kernel's launch overlaps the running one, and a kernel so launched
 // waits for its predecessor's results before it reads or writes anything (pdl_enter is its first
-// statement; a no-op in an ordinary launch).  Microseconds per iteration, ordinary to dependent:
+// statement; a no-op in an ordinary launch).  Such a kernel is resident while its predecessor still
+// writes, so what a kernel of the iteration writes is read with ordinary loads: the read-only path
+// (__ldg, const __restrict__) is specified for data that nobody writes while the kernel runs, and
+// serves only the tables built with the plan.  Microseconds per iteration, ordinary to dependent:
 // dense 128^2 52.6 to 36.5, 256^2 59.0 to 47.9, 701 x 1003 139 to 128, 2048^2 812 to 797; fast
 // transforms 512^2 52.1 to 50.1, 2048^2 102 to 93.7, 4096^2 326 to 314 (Schur).  The tensor-core forms
 // keep the ordinary launch: 256^2 95.0 to 89.9 and 1024^2 130 to 126, but 2048^2 244 to 253 and 4096^2

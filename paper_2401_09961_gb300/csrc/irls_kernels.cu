@@ -166,7 +166,8 @@ __device__ __forceinline__ void emit16(void* r16, void* r16lo, int ld16, int i, 
 // ------------------------------------------------------------------------------------------
 // The two per-iteration kernels work on float4 lanes: a thread owns 4 consecutive columns, a
 // warp 128 and a block of 128 threads 512, so each warp moves 512-byte rows; the next row's
-// loads are issued before the current row's stores (all plane pointers are __restrict__).
+// loads are issued before the current row's stores (the planes a kernel writes are __restrict__;
+// those it only reads are not, see pdl_enter).
 // Columns at or beyond W are zero in every plane; they are computed like the others (their
 // values stay zero) and only the edge masks hh[] exclude the edges that do not exist.
 // ------------------------------------------------------------------------------------------
@@ -191,7 +192,7 @@ constexpr int kSchurRows = 24;
 __device__ __forceinline__ int vec_cols(int W) {
     return (W + kThreads * kVec - 1) / (kThreads * kVec);
 }
-__device__ __forceinline__ void ld4(const float* __restrict__ p, float (&v)[4]) {
+__device__ __forceinline__ void ld4(const float* p, float (&v)[4]) {
     const float4 t = *reinterpret_cast<const float4*>(p);
     v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
 }
@@ -361,17 +362,17 @@ __device__ __forceinline__ void k_direction_pap_body(Planes P, StencilArgs a, De
     const float beta = fresh ? 0.f : (float)st->beta;
     // (selected, not indexed: a batch's planes come from memory, and an indexed copy of them would
     // live in local memory)
-    const float* __restrict__ pUo = cur ? P.pU[1] : P.pU[0];
-    const float* __restrict__ pVvo = cur ? P.pVv[1] : P.pVv[0];
-    const float* __restrict__ pVho = cur ? P.pVh[1] : P.pVh[0];
+    const float* pUo = cur ? P.pU[1] : P.pU[0];
+    const float* pVvo = cur ? P.pVv[1] : P.pVv[0];
+    const float* pVho = cur ? P.pVh[1] : P.pVh[0];
     float* __restrict__ pUn = cur ? P.pU[0] : P.pU[1];
     float* __restrict__ pVvn = cur ? P.pVv[0] : P.pVv[1];
     float* __restrict__ pVhn = cur ? P.pVh[0] : P.pVh[1];
-    const float* __restrict__ zU = P.zU;
-    const float* __restrict__ rVv = P.rVv;
-    const float* __restrict__ rVh = P.rVh;
-    const float* __restrict__ Dv = P.dv;
-    const float* __restrict__ Dh = P.dh;
+    const float* zU = P.zU;
+    const float* rVv = P.rVv;
+    const float* rVh = P.rVh;
+    const float* Dv = P.dv;
+    const float* Dh = P.dh;
     bool hh[kVec];
 #pragma unroll
     for (int e = 0; e < kVec; ++e) hh[e] = j0 + e + 1 < W;
@@ -524,12 +525,12 @@ __device__ __forceinline__ void k_update_body(Planes P, StencilArgs a, DevState*
     const int cur = st->pbuf;
     const float alpha = (float)st->alpha;
     const bool flex = a.flexible != 0;
-    const float* __restrict__ pU = cur ? P.pU[1] : P.pU[0];
-    const float* __restrict__ pVv = cur ? P.pVv[1] : P.pVv[0];
-    const float* __restrict__ pVh = cur ? P.pVh[1] : P.pVh[0];
-    const float* __restrict__ Dv = P.dv;
-    const float* __restrict__ Dh = P.dh;
-    const float* __restrict__ Zu = P.zU;
+    const float* pU = cur ? P.pU[1] : P.pU[0];
+    const float* pVv = cur ? P.pVv[1] : P.pVv[0];
+    const float* pVh = cur ? P.pVh[1] : P.pVh[0];
+    const float* Dv = P.dv;
+    const float* Dh = P.dh;
+    const float* Zu = P.zU;
     float* __restrict__ U = P.U;
     float* __restrict__ Vv = P.Vv;
     float* __restrict__ Vh = P.Vh;
@@ -1282,11 +1283,11 @@ k_schur_direction(Planes P, StencilArgs a, DevState* st, double* partials) {
     const int cur = st->pbuf, nxt = cur ^ 1;
     const bool fresh = st->p_fresh != 0;
     const float beta = fresh ? 0.f : (float)st->beta;
-    const float* __restrict__ pUo = P.pU[cur];
+    const float* pUo = P.pU[cur];
     float* __restrict__ pUn = P.pU[nxt];
-    const float* __restrict__ zU = P.zU;
-    const float* __restrict__ Dv = P.dv;
-    const float* __restrict__ Dh = P.dh;
+    const float* zU = P.zU;
+    const float* Dv = P.dv;
+    const float* Dh = P.dh;
     bool hh[kVec];
 #pragma unroll
     for (int e = 0; e < kVec; ++e) hh[e] = j0 + e + 1 < W;
@@ -1390,10 +1391,10 @@ k_schur_update(Planes P, StencilArgs a, DevState* st, double* partials) {
     const int cur = st->pbuf;
     const float alpha = (float)st->alpha;
     const bool flex = a.flexible != 0;
-    const float* __restrict__ pU = P.pU[cur];
-    const float* __restrict__ Dv = P.dv;
-    const float* __restrict__ Dh = P.dh;
-    const float* __restrict__ Zu = P.zU;
+    const float* pU = P.pU[cur];
+    const float* Dv = P.dv;
+    const float* Dh = P.dh;
+    const float* Zu = P.zU;
     float* __restrict__ U = P.U;
     float* __restrict__ rU = P.rU;
     bool hh[kVec];
