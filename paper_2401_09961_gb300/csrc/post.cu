@@ -200,7 +200,8 @@ k_round_congruent(const float* __restrict__ U, const float* __restrict__ X, size
 }
 
 // alpha = mean(Xu - U) (FP64) into st->aux[1]: four differences and their rounding remainders as
-// one pair, then FP64.
+// one pair, then FP64.  Four pixels with a difference that is not finite, or whose sum could
+// overflow, go to FP64 one by one.
 __global__ void __launch_bounds__(kPostThreads)
 k_shift_mean(const float* __restrict__ U, const float* __restrict__ Xu, size_t n, int vec,
              DevState* st, double* partials) {
@@ -213,8 +214,16 @@ k_shift_mean(const float* __restrict__ U, const float* __restrict__ Xu, size_t n
         float u[4], x[4], d[4], l[4];
         load4(U, i, m, vec, u);
         load4(Xu, i, m, vec, x);
+        bool in_range = true;
 #pragma unroll
-        for (int e = 0; e < 4; ++e) two_sum(x[e], -u[e], d[e], l[e]);
+        for (int e = 0; e < 4; ++e) {
+            two_sum(x[e], -u[e], d[e], l[e]);
+            in_range &= fabsf(d[e]) < 0x1p120f;
+        }
+        if (!in_range) {
+            for (int e = 0; e < m; ++e) s += (double)x[e] - (double)u[e];
+            continue;
+        }
         float a, b, h, e0, e1, e2;
         two_sum(d[0], d[1], a, e0);
         two_sum(d[2], d[3], b, e1);
@@ -226,13 +235,18 @@ k_shift_mean(const float* __restrict__ U, const float* __restrict__ Xu, size_t n
         st->aux[1] = tot[0] / (double)n;
 }
 
-// E = (Xu - U) - alpha (float32), sum of ((Xu - U) - alpha)^2 (pairs, FP64 every four pixels) into
-// st->aux[2]
+// E = (Xu - U) - alpha (float32), sum of ((Xu - U) - alpha)^2 into st->aux[2].  The error of a pixel
+// is the exact difference (a pair) less alpha (three floats), every step error-free and the pair
+// that remains normalised: alpha may be far larger than the errors (images of different offsets),
+// and the second part is squared with the first.  Squares are pairs, FP64 every four pixels.  Four
+// pixels whose largest error is not finite or whose squares could overflow, or lose their
+// remainders below the smallest floats, go to FP64 one by one.
 __global__ void __launch_bounds__(kPostThreads)
 k_shift_error(const float* __restrict__ U, const float* __restrict__ Xu, size_t n, int vec,
               DevState* st, double* partials, float* __restrict__ E) {
     const double alpha = st->aux[1];
-    const float ah = (float)alpha, al = (float)(alpha - (double)ah);
+    const float a1 = (float)alpha, a2 = (float)(alpha - (double)a1);
+    const float a3 = (float)((alpha - (double)a1) - (double)a2);
     double s2 = 0.0;
     const size_t quads = (n + 3) / 4;
     for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < quads;
@@ -242,18 +256,35 @@ k_shift_error(const float* __restrict__ U, const float* __restrict__ Xu, size_t 
         float u[4], x[4], o[4], q[4], r[4];
         load4(U, i, m, vec, u);
         load4(Xu, i, m, vec, x);
+        float most = 0.f;
+        bool in_range = true;
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-            float d, l, p, pe;
+            float d, l, p, w, c0, c1, c2, c3, hi, lo;
             two_sum(x[e], -u[e], d, l);
-            o[e] = __fsub_rn(d, ah);
-            two_sum(d, -ah, p, pe);
-            const float w = __fadd_rn(pe, __fsub_rn(l, al));
+            o[e] = __fsub_rn(d, a1);
+            two_sum(d, -a1, p, c0);
+            two_sum(l, -a2, c1, c2);
+            two_sum(c0, c1, w, c3);
+            two_sum(p, w, hi, lo);
+            two_sum(hi, __fadd_rn(lo, __fsub_rn(__fadd_rn(c2, c3), a3)), p, w);
             two_prod(p, p, q[e], r[e]);
-            r[e] = __fmaf_rn(2.f * p, w, r[e]);
-            if (e >= m) q[e] = r[e] = 0.f;
+            r[e] = __fmaf_rn(2.f * p, w, __fmaf_rn(w, w, r[e]));
+            if (e < m) {
+                in_range &= fabsf(p) < 0x1p60f;
+                most = fmaxf(most, fabsf(p));
+            } else {
+                q[e] = r[e] = 0.f;
+            }
         }
         if (E) store4<float, float4>(E, i, m, vec, o);
+        if (!in_range || (most < 0x1p-45f && most != 0.f)) {
+            for (int e = 0; e < m; ++e) {
+                const double f = ((double)x[e] - (double)u[e]) - alpha;
+                s2 += f * f;
+            }
+            continue;
+        }
         float a, b, h, e0, e1, e2;
         two_sum(q[0], q[1], a, e0);
         two_sum(q[2], q[3], b, e1);
