@@ -173,12 +173,15 @@ int irls_plan_dct_form(irls_plan plan);
 
 /* Tile shapes of the CG direction and update kernels (Alg. 2's two stencil passes per
  * iteration, both bound by HBM bandwidth): image rows per thread block, 8 to 64 for a plan
- * (defaults 24 and 32; batches: one of 8, 16, 24, 32, see irls_batch_set_tiles), or fewer where
- * a small image's launch would otherwise leave SMs idle.  They change the block decomposition, so
- * results change within rounding (the reductions' summation order follows the blocks), never the
- * method.  irls_plan_set_tiles sets them (0 keeps a value;
- * anything outside 8..64 is IRLS_ERR_ARG); irls_plan_get_tiles reads the values in use.
- * irls_plan_autotune times, for each kernel, 8, 16, 24 and 32 rows and the row counts that make
+ * (batches: one of 8, 16, 24, 32, see irls_batch_set_tiles).  The defaults, 24 and 32, stand for
+ * the library's choice: that many rows, or the fewest that still make the launch one wave of
+ * blocks where an image is too small to fill the device with more.  Any other count is used as it
+ * is set.  The shapes change the block decomposition, so results change within rounding (the
+ * reductions' summation order follows the blocks), never the method.  irls_plan_set_tiles sets
+ * them (0 keeps a value; anything outside 8..64 is IRLS_ERR_ARG); irls_plan_get_tiles reads the
+ * values set.
+ * irls_plan_autotune times, for each kernel, 8, 16, 24 and 32 rows (the default count as the
+ * library's choice) and the row counts that make
  * the kernel's launch the fewest whole waves on this device with at most 32 and at most 64 rows
  * a block (when those counts are other ones),
  * on the plan's workspace (ten launches each, after two warm-up launches, CUDA events on

@@ -78,7 +78,8 @@ class Plan:
 
     @property
     def tiles(self):
-        """(direction, update) image rows per block of the CG stencil kernels in use."""
+        """(direction, update) image rows per block set for the CG stencil kernels; the defaults,
+        (24, 32), let the library take fewer on small images."""
         d, u = ctypes.c_int(), ctypes.c_int()
         check(lib().irls_plan_get_tiles(self.handle, ctypes.byref(d), ctypes.byref(u)),
               "irls_plan_get_tiles")

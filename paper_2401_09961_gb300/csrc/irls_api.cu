@@ -527,10 +527,10 @@ void layout_vec_blocks(irls_batch_s* b) {
     for (int t = 0; t < b->T; ++t) {
         TileRec& r = b->recs[t];
         StencilArgs& a = r.a;
-        a.dir_unit = unit_rows(b->dir_rows, a.dir_wave);
-        a.upd_unit = unit_rows(b->upd_rows, a.upd_wave);
-        a.dir_rows = batch_rows(b->dir_rows, a.dir_wave);
-        a.upd_rows = batch_rows(b->upd_rows, a.upd_wave);
+        a.dir_unit = unit_rows(b->dir_rows, kDefaultDirRows, a.dir_wave);
+        a.upd_unit = unit_rows(b->upd_rows, kDefaultUpdRows, a.upd_wave);
+        a.dir_rows = batch_rows(b->dir_rows, a.dir_unit);
+        a.upd_rows = batch_rows(b->upd_rows, a.upd_unit);
         r.vgx = vec_blocks_x(b->W[t]);
         r.vgy = (b->H[t] + a.dir_rows - 1) / a.dir_rows;
         r.ugy = (b->H[t] + a.upd_rows - 1) / a.upd_rows;
@@ -855,22 +855,33 @@ int irls_plan_autotune(irls_plan p, float* h_ms, void* stream) {
         constexpr int kWarm = 2, kReps = 10;
         // candidates: the fixed row counts, then for each kernel the counts that make its
         // launch the fewest whole waves with at most 32 and at most 64 rows a block (where they
-        // are not among the others)
-        int cand[2][6];
+        // are not among the others).  rows: what a candidate launches (the default may take fewer)
+        int cand[2][6], rows[2][6];
         int ncand[2];
         for (int k = 0; k < 2; ++k) {
-            for (int i = 0; i < 4; ++i) cand[k][i] = kTileRows[i];
+            const int dflt = k == 0 ? kDefaultDirRows : kDefaultUpdRows;
+            const int wave = k == 0 ? a.dir_wave : a.upd_wave;
+            for (int i = 0; i < 4; ++i) {
+                cand[k][i] = kTileRows[i];
+                rows[k][i] = unit_rows(kTileRows[i], dflt, wave);
+            }
             ncand[k] = 4;
             for (int cap : {32, kMaxTileRows}) {
                 const int w = wave_rows(k, p->H, p->W, cap);
                 bool seen = (w == 0);
-                for (int i = 0; i < ncand[k]; ++i) seen |= (cand[k][i] == w);
-                if (!seen) cand[k][ncand[k]++] = w;
+                for (int i = 0; i < ncand[k]; ++i) seen |= (rows[k][i] == w);
+                if (!seen) cand[k][ncand[k]] = rows[k][ncand[k]] = w, ++ncand[k];
             }
         }
         float ms[2][6];
         for (int k = 0; k < 2; ++k)
             for (int i = 0; i < ncand[k]; ++i) {
+                // a launch that was timed already, as another candidate
+                const int* same = std::find(rows[k], rows[k] + i, rows[k][i]);
+                if (same != rows[k] + i) {
+                    ms[k][i] = ms[k][same - rows[k]];
+                    continue;
+                }
                 StencilArgs b = a;
                 if (k == 0) b.dir_rows = cand[k][i];
                 else b.upd_rows = cand[k][i];

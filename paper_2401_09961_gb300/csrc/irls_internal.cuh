@@ -115,8 +115,8 @@ struct StencilArgs {
     int rw_rows, fin_rows;
     int sdir_rows, supd_rows;   // U-only system's direction and update kernels (0: 24)
     // rows that make the direction and update launches of this image one wave (0: unknown): a
-    // launch sums its inner products in units of min(dir_rows, dir_wave) rows, and a single
-    // image's blocks hold one unit (see unit_rows)
+    // launch sums its inner products in units of unit_rows rows, and a single image's blocks hold
+    // one unit
     int dir_wave, upd_wave;
     int dir_unit, upd_unit;     // batches: rows of a summation unit (dir_rows, upd_rows: of a block)
     // single-image CG runs: where the update kernels report to the host (pinned memory; null: no
@@ -127,19 +127,20 @@ struct StencilArgs {
     int full;  // float32 dense products at full size (host; a taped solve or its adjoint)
 };
 
-// Rows of a summation unit for a tile of `rows` rows and a one-wave count of `wave` rows, and the
-// whole units a batch's block holds.  Small images leave most SMs idle at the tile's rows, and a
+// Rows of a summation unit for a tile of `rows` rows (`dflt`: the kernel's default) and a one-wave
+// count of `wave` rows, and the whole units a batch's block holds.  The default stands for the
+// library's choice, at most one wave's rows; any other count was set by the caller and holds as it
+// is.  Small images leave most SMs idle at the tile's rows, and a
 // block's rows are a serial chain of about a microsecond each: blocks of the fewest rows that
 // still run at once are as fast as the chip allows.  In a batch the other images fill the chip,
 // and blocks of several units save the halo rows and the block ends.  Measured (us of one launch,
 // direction / update): 1024^2 at 12 rows 30 / 28, at 8 24 / 24, at the one-wave 3 / 4 rows 18 / 22,
 // at 1 28 / 42; 256^2 at 8 rows 22 / 18, at 1 (one wave) 10 / 14; 2048^2 at 24 / 32 rows 53 / 68, at
 // the one-wave 11 / 14 49 / 59.
-inline int unit_rows(int rows, int wave) { return wave > 0 && wave < rows ? wave : rows; }
-inline int batch_rows(int rows, int wave) {
-    const int u = unit_rows(rows, wave);
-    return rows / u * u;
+inline int unit_rows(int rows, int dflt, int wave) {
+    return rows == dflt && wave > 0 && wave < rows ? wave : rows;
 }
+inline int batch_rows(int rows, int unit) { return rows / unit * unit; }
 
 // Image rows per block the CG direction and update kernels are built for, and the defaults
 // (measured fastest at 4096 x 4096).

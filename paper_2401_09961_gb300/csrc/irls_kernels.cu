@@ -1786,14 +1786,14 @@ cudaError_t launch_reweight_residual(const Planes& P, const StencilArgs& a, DevS
 cudaError_t launch_direction_pap(const Planes& P, const StencilArgs& a, DevState* st,
                                  double* partials, cudaStream_t s) {
     StencilArgs b = a;
-    b.dir_rows = unit_rows(rows_or(a.dir_rows, kDirRows), a.dir_wave);
+    b.dir_rows = unit_rows(rows_or(a.dir_rows, kDirRows), kDirRows, a.dir_wave);
     return launch_rows<DirK>(b.dir_rows, a.H, a.W, s, P, b, st, partials);
 }
 
 cudaError_t launch_update(const Planes& P, const StencilArgs& a, DevState* st, double* partials,
                           cudaStream_t s) {
     StencilArgs b = a;
-    b.upd_rows = unit_rows(rows_or(a.upd_rows, kUpdRows), a.upd_wave);
+    b.upd_rows = unit_rows(rows_or(a.upd_rows, kUpdRows), kUpdRows, a.upd_wave);
     return launch_rows<UpdK>(b.upd_rows, a.H, a.W, s, P, b, st, partials);
 }
 
