@@ -453,7 +453,11 @@ __device__ __forceinline__ void k_direction_pap_body(Planes P, StencilArgs a, De
             for (int e = 0; e < 4; ++e) {
                 const float yh = hh[e] ? (pr[e] - cu[e] - cvh[e]) : 0.f;
                 const float yv = hv ? (nu[e] - cu[e] - cvv[e]) : 0.f;
-                row += it * (yh * yh + yv * yv) + cdv[e] * cvv[e] * cvv[e] + cdh[e] * cvh[e] * cvh[e];
+                // written out: the same roundings in every instance of this kernel
+                const float q = __fmaf_rn(yh, yh, __fmul_rn(yv, yv));
+                const float dv = __fmul_rn(__fmul_rn(cdv[e], cvv[e]), cvv[e]);
+                row = __fadd_rn(row, __fmaf_rn(__fmul_rn(cdh[e], cvh[e]), cvh[e],
+                                               __fmaf_rn(it, q, dv)));
             }
             acc.add(row);
         }
@@ -613,8 +617,12 @@ __device__ __forceinline__ void k_update_body(Planes P, StencilArgs a, DevState*
                                                                       __fmul_rn(n0[e], n0[e]))));
                 pru2 = __fmaf_rn(n0[e], n0[e], pru2);
                 psu = __fadd_rn(psu, n0[e]);
-                przv += n1[e] * n1[e] * iv + n2[e] * n2[e] * ih;
-                if (flex) przo += n0[e] * z[e] + (n1[e] * r1[e]) * iv + (n2[e] * r2[e]) * ih;
+                przv = __fadd_rn(przv, __fmaf_rn(__fmul_rn(n1[e], n1[e]), iv,
+                                                 __fmul_rn(__fmul_rn(n2[e], n2[e]), ih)));
+                if (flex) {
+                    const float v = __fmaf_rn(n0[e], z[e], __fmul_rn(__fmul_rn(n1[e], r1[e]), iv));
+                    przo = __fadd_rn(przo, __fmaf_rn(__fmul_rn(n2[e], r2[e]), ih, v));
+                }
             }
             rr.add(prr);
             ru2.add(pru2);
