@@ -776,19 +776,24 @@ void dct_release(DctPlan& d) {
 cudaError_t dct_full_setup(DctPlan& d, cudaStream_t s) {
     if (d.full_mem || d.fft || d.prec != IRLS_PREC_FP32) return cudaSuccess;
     const size_t n = (size_t)d.Hp * d.Hp, m = d.H != d.W ? (size_t)d.Wp * d.Wp : 0;
-    cudaError_t e = cudaMalloc(&d.full_mem, 2 * (n + m) * sizeof(float));
+    void* mem = nullptr;
+    cudaError_t e = cudaMalloc(&mem, 2 * (n + m) * sizeof(float));
     if (e != cudaSuccess) {
         cudaGetLastError();
-        d.full_mem = nullptr;
         return e;
     }
-    d.PN = static_cast<float*>(d.full_mem);
+    d.PN = static_cast<float*>(mem);
     d.PNT = d.PN + n;
     d.PM = m ? d.PNT + n : d.PN;
     d.PMT = m ? d.PM + m : d.PNT;
     k_build_full<<<1024, 256, 0, s>>>(d.PN, d.PNT, d.H, d.Hp);
     if (m) k_build_full<<<1024, 256, 0, s>>>(d.PM, d.PMT, d.W, d.Wp);
-    return cudaGetLastError();
+    if ((e = cudaGetLastError()) != cudaSuccess) {
+        cudaFree(mem);
+        return e;
+    }
+    d.full_mem = mem;   // (set last: a plan that has it has the bases)
+    return cudaSuccess;
 }
 cudaError_t dct_reset(const DctPlan& d, cudaStream_t s) { return umma_dct_reset(d, s); }
 bool dct_stall(DctPlan& d, int on) { return umma_dct_stall(d, on); }
