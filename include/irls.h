@@ -323,7 +323,13 @@ int irls_batch_autotune(irls_batch batch, float* h_ms, void* stream);
  * planes allocated by the library.  Arguments as in irls_unwrap_ex (no restart point).
  * *tape receives the record; release it with irls_tape_free.  The plan must outlive the tape;
  * other solves on the plan between recording and the backward call are allowed (the tape
- * keeps its own copies).  Synchronous like irls_unwrap_ex. */
+ * keeps its own copies).  Synchronous like irls_unwrap_ex.
+ * With the float32 dense products (IRLS_PREC_FP32, not IRLS_DCT_FFT) a recorded solve and its
+ * adjoint run the preconditioner's products at full size, irls_unwrap_ex as quadrants of half
+ * the size: U is the same within rounding, not bit for bit.  The plan's first such recorded solve
+ * allocates their bases (2 H^2 + 2 W^2 floats, sides rounded up to multiples of 128, half of it
+ * for a square; kept until the plan is destroyed; IRLS_ERR_OOM when they do not fit).  The
+ * backward call allocates nothing. */
 int irls_unwrap_forward_record(irls_plan plan, const float* d_X, const float* d_coherence,
                                const float* d_Cv, const float* d_Ch, float* d_U, irls_tape* tape,
                                irls_stats* h_stats, void* stream);

@@ -774,7 +774,7 @@ void dct_release(DctPlan& d) {
 // The full-size bases of the float32 dense form, on the first solve of a plan that needs them
 // (kept with the plan).  Nothing for the other forms.
 cudaError_t dct_full_setup(DctPlan& d, cudaStream_t s) {
-    if (d.full_mem || d.fft || d.prec != IRLS_PREC_FP32) return cudaSuccess;
+    if (d.full_mem || !dct_runs_full(d)) return cudaSuccess;
     const size_t n = (size_t)d.Hp * d.Hp, m = d.H != d.W ? (size_t)d.Wp * d.Wp : 0;
     void* mem = nullptr;
     cudaError_t e = cudaMalloc(&mem, 2 * (n + m) * sizeof(float));

@@ -194,6 +194,7 @@ struct irls_plan_s {
 struct irls_tape_s {
     irls_plan_s* plan = nullptr;
     int H = 0, W = 0, ld = 0, K = 0, has_coh = 0;
+    int full = 0;   // recorded with the full-size float32 products, which its adjoint then runs too
     float tau = 0.f, delta = 0.f;
     char* mem = nullptr;
     size_t plane_bytes = 0;
@@ -1005,6 +1006,7 @@ int irls_unwrap_forward_record(irls_plan p, const float* X, const float* coh, co
         } else {
             ck(e);
         }
+        t->full = dct_runs_full(p->dct);
         size_t q = 0;
         t->Gv = f[q++]; t->Gh = f[q++]; t->Cv = f[q++]; t->Ch = f[q++];
         t->Gbv = f[q++]; t->Gbh = f[q++]; t->Cbv = f[q++]; t->Cbh = f[q++];
@@ -1040,11 +1042,7 @@ int irls_unwrap_backward(irls_tape t, const float* dLdU, float* dLdX, float* dLd
     try {
         DeviceGuard g(p->dev);
         StencilArgs a = make_args(p);
-        a.full = 1;
-        if (cudaError_t e = dct_full_setup(p->dct, s); e == cudaErrorMemoryAllocation)
-            return IRLS_ERR_OOM;
-        else
-            ck(e);
+        a.full = t->full;   // (its plan has the bases: nothing is allocated here)
         DevState* st = p->st;
         const size_t pb = t->plane_bytes;
         ck(cudaMemsetAsync(st, 0, sizeof(DevState), s));

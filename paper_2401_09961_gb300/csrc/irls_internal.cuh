@@ -332,6 +332,8 @@ cudaError_t dct_setup(DctPlan& d, int H, int W, int prec, float tau, char* mem);
 // receives error flags; with reduce_rho the last GEMM also forms rho = r_U^T z_U + st->rz_v
 // and the next beta (Alg. 2).  With skip_if_done the launches return at once once CG stopped.
 void dct_release(DctPlan& d);
+// the float32 dense form's full-size bases, for a plan whose options run that form
+inline bool dct_runs_full(const DctPlan& d) { return !d.fft && d.prec == IRLS_PREC_FP32; }
 cudaError_t dct_full_setup(DctPlan& d, cudaStream_t s);
 // zeroes the folded form's launch counters (recovery after a launch that timed out)
 cudaError_t dct_reset(const DctPlan& d, cudaStream_t s);
