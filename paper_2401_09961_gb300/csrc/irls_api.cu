@@ -7,11 +7,13 @@
 // kAhead ahead of the one the device last reported complete (a word in pinned memory), so the GPU
 // neither idles waiting for the host nor runs through many launches after the stop.
 #include <algorithm>
+#include <chrono>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
 #include <mutex>
 #include <new>
+#include <thread>
 #include <vector>
 
 #include "irls_internal.cuh"
@@ -318,16 +320,28 @@ int fetch_stats(irls_plan_s* p, cudaStream_t s, irls_stats* stats) {
     return p->h_flag[0];
 }
 
+// How the process asked for waits to be done (cudaSetDeviceFlags): the flags of this device.
+unsigned wait_schedule() {
+    unsigned f = 0;
+    ck(cudaGetDeviceFlags(&f));
+    return f & cudaDeviceScheduleMask;
+}
+
 // Waits until the device is at most kAhead iterations behind the `issued` ones of run `epoch`;
-// true when the run has stopped.
-bool run_stopped(irls_plan_s* p, unsigned epoch, int issued, cudaStream_t s) {
+// true when the run has stopped.  The wait sleeps where the process asked for blocking waits (the
+// sleeps, about 70 us with the scheduler's slack, fit the iterations in flight), spins where it
+// asked for spinning, and else gives its core to any other thread that is ready.
+bool run_stopped(irls_plan_s* p, unsigned epoch, int issued, unsigned schedule, cudaStream_t s) {
     const volatile unsigned long long* w = p->h_prog;
+    const bool blocking = schedule == cudaDeviceScheduleBlockingSync;
     for (unsigned spin = 1;; ++spin) {
         const unsigned long long v = *w;
         const bool ours = (unsigned)(v >> 32) == epoch;
         if (ours && (v >> 31 & 1)) return true;
         if (issued - (ours ? (int)(v & 0x7fffffffu) : 0) <= kAhead) return false;
-        if (spin % 1024 == 0) {
+        if (blocking) std::this_thread::sleep_for(std::chrono::microseconds(20));
+        else if (schedule != cudaDeviceScheduleSpin) std::this_thread::yield();
+        if (spin % (blocking ? 64 : 1024) == 0) {
             // nothing left in flight: an error, or a run that the report does not cover
             const cudaError_t e = cudaStreamQuery(s);
             if (e == cudaErrorNotReady) continue;
@@ -350,6 +364,7 @@ void run_cg(irls_plan_s* p, StencilArgs a, DevState* st, cudaStream_t s,
     const bool schur = schur_system || p->opts.system == IRLS_SYS_SCHUR;
     a.progress = p->h_prog;
     a.epoch = ++p->epoch;
+    const unsigned schedule = wait_schedule();
     for (int issued = 0; issued < a.cg_max;) {
         t0 = pf.begin(s);
         if (schur) ck(launch_schur_direction(p->P, a, st, p->partials, s));
@@ -362,7 +377,7 @@ void run_cg(irls_plan_s* p, StencilArgs a, DevState* st, cudaStream_t s,
         t0 = pf.begin(s);
         ck(dct_apply(p->dct, p->P.rU, p->P.zU, p->ld, st, 1, a, p->partials, 1, s));
         pf.end(PC_DCT, t0, s);
-        if (run_stopped(p, a.epoch, ++issued, s)) break;
+        if (run_stopped(p, a.epoch, ++issued, schedule, s)) break;
     }
     if (pf.on) {
         ck(cudaStreamSynchronize(s));
