@@ -378,6 +378,13 @@ void run_cg(irls_plan_s* p, StencilArgs a, DevState* st, cudaStream_t s,
         ck(dct_apply(p->dct, p->P.rU, p->P.zU, p->ld, st, 1, a, p->partials, 1, s));
         pf.end(PC_DCT, t0, s);
         if (run_stopped(p, a.epoch, ++issued, schedule, s)) break;
+        // the profiler's pairs of iterations that are over (the last kAhead and two more stay)
+        constexpr size_t kKeep = 3 * (kAhead + 2);
+        if (pf.pend.size() >= 4 * kKeep) {
+            const size_t n = pf.pend.size() - kKeep;
+            ck(cudaEventSynchronize(pf.pend[n - 1].b));
+            pf.drain(n);
+        }
     }
     if (pf.on) {
         ck(cudaStreamSynchronize(s));
