@@ -209,8 +209,8 @@ int irls_debug_stall_fold(irls_plan plan, int on);
  * non-NULL and rec_items >= the item count, also IRLS_FOLD_SCHED_INTS ints per item in list
  * order:
  *   0 stage (0-3), 1 image, 2 tile within its problem, 3 first output row, 4 first column,
- *   5 columns, 6 k-blocks per operand set, 7 two operand sets, 8 half of a stage-3 tile (a
- *   halved stage-2 tile shows by its columns),
+ *   5 columns, 6 k-blocks per operand set, 7 two operand sets, 8 half of a tile: 1 at the end
+ *   of stage 3, 2 in stage 2 (0: a whole tile),
  *   9 counter the tile completes (-1: none; each CTA of the pair adds one),
  *   10 dependency count, 11-18 counters waited for (-1 unused), 19-26 counts waited for,
  *   27 last tile of its pair in the image's stage-2 run, 28 r^T z slots of the image,

@@ -2465,7 +2465,7 @@ bool fold_schedule(const int* H, const int* W, int T, int pairs, int& n_items, i
         r[5] = (f.half || k == 0) ? 128 : 256;
         r[6] = f.nkb;
         r[7] = f.dual;
-        r[8] = k == 3 ? f.half : 0;   // the tail's halves
+        r[8] = !f.half ? 0 : k == 3 ? 1 : 2;   // the tail's halves, a stage's
         r[9] = f.sig;
         r[10] = f.ndep;
         for (int d = 0; d < kMaxDeps; ++d) {
