@@ -542,12 +542,12 @@ cudaError_t fold_products(const float* R, int ldr, float* Z, int ldz, int H, int
 // one-wave rows and the dependent launches).
 constexpr int kFullTile = 128;
 
-enum Epi : int { EPI_TRANS = 0, EPI_EIG = 1, EPI_ZU = 2, EPI_ZU_RHO = 3 };
+enum Epi : int { EPI_TRANS = 0, EPI_EIG = 1, EPI_ZU_RHO = 2 };
 
 struct EpiArgs {
     float* C;          // output
     int ldc;
-    int vm, vn;        // valid extents (EPI_EIG: W, H; EPI_ZU: H, W)
+    int vm, vn;        // valid extents (EPI_EIG: W, H; EPI_ZU_RHO: H, W)
     const float* lam_m;
     const float* lam_n;
     float scale;       // tau (EPI_EIG)
@@ -646,7 +646,7 @@ k_gemm_tn_f32(const float* __restrict__ A, int lda, int a_rows, const float* __r
             } else {
                 if (m < ep.vm && n < ep.vn) {
                     ep.C[(size_t)m * ep.ldc + n] = v;
-                    if constexpr (EPI == EPI_ZU_RHO) row += ep.rU[(size_t)m * ep.ldc + n] * v;
+                    row += ep.rU[(size_t)m * ep.ldc + n] * v;
                 }
             }
         }
@@ -686,9 +686,9 @@ cudaError_t full_gemm(const float* A, int lda, int a_rows, const float* B, int l
     return cudaGetLastError();
 }
 
+// (always with rho: only CG runs take these products)
 cudaError_t full_products(const DctPlan& d, const float* rU, float* zU, int ld, DevState* st,
-                          int reduce_rho, int flexible, double* partials, int skip,
-                          cudaStream_t s) {
+                          int flexible, double* partials, int skip, cudaStream_t s) {
     const int H = d.H, W = d.W, Hp = d.Hp, Wp = d.Wp;
     cudaError_t e;
     EpiArgs ep{};
@@ -710,8 +710,7 @@ cudaError_t full_products(const DctPlan& d, const float* rU, float* zU, int ld, 
     if (e != cudaSuccess) return e;
     // stage 4: Z[i][j] = sum_l T1[i][l] PM[j][l]
     ep.C = zU; ep.ldc = ld; ep.vm = H; ep.vn = W; ep.rU = rU;
-    return reduce_rho ? full_gemm<EPI_ZU_RHO>(d.T1, Wp, Hp, d.PM, Wp, Hp, Wp, W, ep, skip, s)
-                      : full_gemm<EPI_ZU>(d.T1, Wp, Hp, d.PM, Wp, Hp, Wp, W, ep, skip, s);
+    return full_gemm<EPI_ZU_RHO>(d.T1, Wp, Hp, d.PM, Wp, Hp, Wp, W, ep, skip, s);
 }
 
 }  // namespace
@@ -805,8 +804,7 @@ cudaError_t dct_apply(const DctPlan& d, const float* rU, float* zU, int ld, DevS
     if (d.prec != IRLS_PREC_FP32)
         return umma_dct_apply(d, rU, zU, ld, st, reduce_rho, a, partials, skip_if_done, s, src,
                               ld_src);
-    if (a.full)
-        return full_products(d, rU, zU, ld, st, reduce_rho, a.flexible, partials, skip_if_done, s);
+    if (a.full) return full_products(d, rU, zU, ld, st, a.flexible, partials, skip_if_done, s);
     QuadArgs base{};
     base.st = st;
     base.partials = partials;

@@ -271,11 +271,12 @@ __device__ __forceinline__ void inv_pair(float* s, int f, int k, float ya_k, flo
     if (k != N - k) L::st(s, f, N - k, make_float2(pa.x + pb.y, pa.y - pb.x));
 }
 
-// Launch shapes: one thread per radix-16 butterfly of the block's NF transforms.  Rows: the
-// pairs of rows of up to 4096 elements a block; columns: strips of 4 to 32 columns.
+// Rows of 16000 and 16384 elements (below, quads): one pair of rows a block, one thread per radix-16
+// butterfly of its transform.
 template <int N>
 struct RowCfg {
-    static constexpr int NF = (4096 / N) < 1 ? 1 : ((4096 / N) > 16 ? 16 : 4096 / N);
+    static_assert(N == 16000 || N == 16384, "the others run quads");
+    static constexpr int NF = 1;
     static constexpr int T = (N * NF / 16 + 31) / 32 * 32;   // whole warps
     using L = PairL<N, NF>;
     static constexpr size_t SMEM = (size_t)L::FLOATS * sizeof(float) + TwN<N>::PADDED * sizeof(float2);

@@ -177,7 +177,7 @@ struct irls_plan_s {
     DevState* st = nullptr;
     double* partials = nullptr;
     DctPlan dct{};
-    int* h_flag = nullptr;     // pinned, 2 slots
+    int* h_flag = nullptr;     // pinned: a status word read back
     double* h_pair = nullptr;  // pinned, 2 doubles: H_delta values read by the Sec. 4.3 rule
     unsigned long long* h_prog = nullptr;   // pinned: the update kernels' progress reports
     unsigned epoch = 0;                     // CG runs issued
@@ -246,7 +246,7 @@ StencilArgs make_args(const irls_plan_s* p) {
 // Folded preconditioner on or off for the given options; false when IRLS_DCT_FOLDED is asked for
 // and the plan has no folded form (a shape or precision that does not allow it).
 bool select_dct_form(irls_plan_s* p, const irls_opts& o) {
-    // the fast-transform form computes in float32 and takes power-of-two sides
+    // the fast-transform form computes in float32 and takes the lengths its kernels are built for
     if (o.dct_form == IRLS_DCT_FFT) {
         if (o.precision != IRLS_PREC_FP32 || !p->dct.fft_ready) return false;
         p->dct.fft = 1;
@@ -797,7 +797,7 @@ int irls_plan_create(int H, int W, const irls_opts* opts, irls_plan* out) {
             destroy_plan(p);
             return IRLS_ERR_UNSUPPORTED;
         }
-        ck(cudaHostAlloc(&p->h_flag, 2 * sizeof(int), cudaHostAllocDefault));
+        ck(cudaHostAlloc(&p->h_flag, sizeof(int), cudaHostAllocDefault));
         ck(cudaHostAlloc(&p->h_pair, 2 * sizeof(double), cudaHostAllocDefault));
         ck(cudaHostAlloc(&p->h_prog, sizeof(unsigned long long), cudaHostAllocMapped));
         *p->h_prog = 0;
