@@ -1534,9 +1534,10 @@ k_schur_recover_v(Planes P, StencilArgs a) {
 // One product with A on the caller's arrays: q_U = (S^T y_v + y_h T^T) / tau, q_V = D V - y / tau
 // with the update kernel's arithmetic (hi + lo pairs of the cancelling terms).  A thread owns one
 // column and marches down `rows` rows, the next row's loads issued before this row's stores; rows
-// of any pitch and alignment.  Bound by memory: 32 bytes a pixel and 12 a strip's end row.  2047 x
-// 1999: 35 us, host call included (through the plan's planes and the update kernel, with their
-// eleven memsets and eight copies: 266 us).
+// of any pitch and alignment.  32 bytes a pixel and 12 a strip's end row are 19 us at 2047 x 1999 and
+// the memory rate; the edge arrays' odd pitch (W - 1) makes the seven streams element-wise loads,
+// which take the 35 us (3.75 TB/s) it runs in, host call included (through the plan's planes and the
+// update kernel, with their eleven memsets and eight copies: 266 us).
 // ------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(kThreads)
 k_apply_A(const float* __restrict__ U, const float* __restrict__ Vv, const float* __restrict__ Vh,
@@ -1811,7 +1812,8 @@ cudaError_t launch_schur_reweight(const Planes& P, const StencilArgs& a, DevStat
     return cudaGetLastError();
 }
 
-// U-only CG kernels: the plan's whole-wave row counts (a.sdir_rows, a.supd_rows), else 24 rows
+// U-only CG kernels: the plan's row counts (aux_rows: one wave's, whole waves of up to 64 rows, or 32);
+// 24 where the arguments carry none
 cudaError_t launch_schur_direction(const Planes& P, const StencilArgs& a, DevState* st,
                                    double* partials, cudaStream_t s) {
     const int rows = a.sdir_rows > 0 ? a.sdir_rows : kSchurRows;

@@ -240,7 +240,9 @@ k_shift_mean(const float* __restrict__ U, const float* __restrict__ Xu, size_t n
 // that remains normalised: alpha may be far larger than the errors (images of different offsets),
 // and the second part is squared with the first.  Squares are pairs, FP64 every four pixels.  Four
 // pixels whose largest error is not finite or whose squares could overflow, or lose their
-// remainders below the smallest floats, go to FP64 one by one.
+// remainders below the smallest floats, go to FP64 one by one.  (Without the third float, the second
+// normalisation and the range check the two calls at 4096^2 take 283 us instead of 292, but an offset
+// of 1000 rad over 1e-3 rad of noise puts rms off by 2e-4.)
 __global__ void __launch_bounds__(kPostThreads)
 k_shift_error(const float* __restrict__ U, const float* __restrict__ Xu, size_t n, int vec,
               DevState* st, double* partials, float* __restrict__ E) {
