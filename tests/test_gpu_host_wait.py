@@ -23,9 +23,12 @@ X = torch.randn(2048, 2048, device="cuda", generator=torch.Generator("cuda").man
 with irls.Plan(2048, 2048, precision="bf16x3", tau=1e-2, delta=1e-3, outer_iters=2, cg_tol=0.0,
                cg_max_iter=400) as p:
     p.unwrap(X)
-    c, t = time.thread_time(), time.perf_counter()
-    U, st = p.unwrap(X)
-    print("TIMES", json.dumps([time.thread_time() - c, time.perf_counter() - t, sum(st["cg_iters"])]))
+    runs = []
+    for _ in range(3):
+        c, t = time.thread_time(), time.perf_counter()
+        U, st = p.unwrap(X)
+        runs.append([time.perf_counter() - t, time.thread_time() - c, sum(st["cg_iters"])])
+    print("TIMES", json.dumps(min(runs)))
 """
 
 
@@ -41,9 +44,9 @@ def test_blocking_waits_leave_the_core():
     is the launches, about 5 a 250 us iteration.  A spin takes the whole time."""
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
-    cpu, wall, its = times(4)
+    wall, cpu, its = times(4)   # the quickest of three runs
     assert its == 800
     assert cpu <= 0.6 * wall, (cpu, wall)
-    spin_cpu, spin_wall, _ = times(1)
-    # and the sleeps fit the iterations in flight: the solve takes no longer
-    assert wall <= 1.1 * spin_wall, (wall, spin_wall)
+    spin_wall, _, _ = times(1)
+    # and the sleeps fit the iterations in flight (a 70 us sleep after every 250 us one: 1.28)
+    assert wall <= 1.15 * spin_wall, (wall, spin_wall)
